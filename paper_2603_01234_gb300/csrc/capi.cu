@@ -230,7 +230,7 @@ struct nep_model {
     Buf partial, partial2, counters, gcounters, totals, flags, thermo, sample_index;
     Buf acc;  // FP32 form: force and virial fixed-point lines, thread virial sums (acc_bytes)
     bool eval_per_bead = false;  // the evaluation in progress returns per-particle virials
-    bool cells_dirty = true;     // the cell counters may be non-zero (new buffer, or a build that failed)
+    bool cells_dirty = true;     // the cell counters may be non-zero (a build that failed)
     Buf types_d, pos_d, vel_d, force_d, virial_d, site_d, force_tmp, totals_tmp;
     Buf noise_d, bussi;  // thermostat: random numbers of the call; [step, alpha] words
     Buf md_virial, md_site, heat, heat_rows;  // HNEMD: per-particle W_i and U_i; acc[6] + counter; rows
@@ -461,8 +461,10 @@ int ensure_lists(nep_model* m, int n)
 
 int ensure_cells(nep_model* m, int ncell)
 {
-    // the scan leaves the cell and fill counters zero for the next build; a new
-    // buffer starts with anything in it, so the next build clears them first
+    // the scan leaves the counters of the cells it covers zero for the next build.  A
+    // new buffer starts with anything in it and a failed build may leave counts behind,
+    // so both are cleared over their whole capacity: a buffer grows by a quarter at
+    // least, and a later grid may reach cells that this one does not
     const void* c0 = m->cell_count.p;
     const void* f0 = m->cell_fill.p;
     const void* b0 = m->block_off.p;
@@ -471,7 +473,13 @@ int ensure_cells(nep_model* m, int ncell)
     NEP_TRY(m->block_off.ensure(sizeof(int) * (kScanItems + 1)));
     NEP_TRY(m->cell_fill.ensure(sizeof(int) * ncell));
     NEP_TRY(m->cell_start.ensure(sizeof(int) * (ncell + 1)));
-    if (m->cell_count.p != c0 || m->cell_fill.p != f0 || m->block_off.p != b0) m->cells_dirty = true;
+    if (m->cells_dirty || m->cell_count.p != c0 || m->cell_fill.p != f0 || m->block_off.p != b0) {
+        m->cells_dirty = true;
+        NEP_CUDA(cudaMemsetAsync(m->cell_count.p, 0, m->cell_count.cap, m->cur));
+        NEP_CUDA(cudaMemsetAsync(m->cell_fill.p, 0, m->cell_fill.cap, m->cur));
+        NEP_CUDA(cudaMemsetAsync(m->block_off.p, 0, m->block_off.cap, m->cur));
+        m->cells_dirty = false;
+    }
     return NEP_OK;
 }
 
@@ -506,7 +514,7 @@ template <typename real>
 int run_cells(nep_model* m, const Plan& p, const int* types_d, const double* pos_d)
 {
     cudaError_t e = launch_cell_build<real>(
-        d_counts(p), p.n_cap, p.items_cap, p.ncell_cap, m->cells_dirty, false, d_items(p), d_reqs(p), d_models<real>(p),
+        d_counts(p), p.n_cap, p.items_cap, p.ncell_cap, false, false, d_items(p), d_reqs(p), d_models<real>(p),
         pos_d, types_d, m->cell_of.as<int>(), m->rec_user.as<PosRec<real>>(), m->cell_count.as<int>(),
         m->cell_local.as<int>(), m->block_off.as<int>(), m->cell_fill.as<int>(), m->perm_tmp.as<int>(),
         m->perm.as<int>(), m->cell_start.as<int>(), m->cell_s.as<int>(), m->rec_s.as<PosRec<real>>(),
@@ -515,21 +523,16 @@ int run_cells(nep_model* m, const Plan& p, const int* types_d, const double* pos
         m->cells_dirty = true;
         return fail(NEP_ERR_CUDA, std::string("cell build: ") + cudaGetErrorString(e));
     }
-    m->cells_dirty = false;
     return NEP_OK;
 }
 
 // The MD step's opening (kicks, drift, binning in one kernel) and the rest of the
-// cell build.  Counters that may be dirty are cleared before the binning counts.
+// cell build.
 template <typename real>
 int run_kick_drift_cells(nep_model* m, const Plan& p, const int* types_d, const double* inv_m_acc, int n_kicks,
                          double half_dt, double dt, double* pos, double* vel, const double* force,
                          cudaEvent_t* ev = nullptr)
 {
-    if (m->cells_dirty) {
-        NEP_CUDA(cudaMemsetAsync(m->cell_count.p, 0, sizeof(int) * p.ncell_cap, m->cur));
-        NEP_CUDA(cudaMemsetAsync(m->cell_fill.p, 0, sizeof(int) * p.ncell_cap, m->cur));
-    }
     TypeTable tt;
     for (int k = 0; k < kMdMaxTypes; ++k) tt.v[k] = k < m->T ? inv_m_acc[k] : 0.0;
     cudaError_t e = launch_kick_drift_bin<real>(d_counts(p), p.items_cap, d_items(p), d_reqs(p), d_models<real>(p),
@@ -548,7 +551,6 @@ int run_kick_drift_cells(nep_model* m, const Plan& p, const int* types_d, const 
         m->cells_dirty = true;
         return fail(NEP_ERR_CUDA, std::string("kick/drift + cell build: ") + cudaGetErrorString(e));
     }
-    m->cells_dirty = false;
     return NEP_OK;
 }
 
@@ -737,15 +739,13 @@ std::vector<unsigned char> eval_graph_key(const nep_model* m, const Plan& p, con
 // The evaluation pipeline, replayed from a captured CUDA graph when one matches
 // (cached on the handle, a few at a time).  Batches are planned with rounded
 // capacities and the kernels read the actual sizes from the device, so batches of
-// similar size share one graph.  A build whose cell counters may be dirty runs
-// eagerly (it clears them first).
+// similar size share one graph.
 template <typename real>
 int eval_launch(nep_model* m, const Plan& p, const int* types_d, const double* pos_d, double* force,
                 double* virial, double* site, double* totals)
 {
     NEP_TRY(ensure_plan_workspace(m, p));
     m->eval_per_bead = virial != nullptr;
-    if (m->cells_dirty) return eval_pipeline<real>(m, p, types_d, pos_d, force, virial, site, totals);
     const void* io[] = {types_d, pos_d, force, virial, site, totals};
     std::vector<unsigned char> key = eval_graph_key<real>(m, p, io, 6);
     for (size_t k = 0; k < m->eval_graphs.size(); ++k)
