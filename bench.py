@@ -512,7 +512,7 @@ def run_ours(args):
     if not args.quick:
         # BF16-weight network form
         bf16 = variant_leg(model, "bf16", "f32 + bf16 W0",
-                           "BF16 hidden-layer weights, tensor-core network products; timed like the headline")
+                           "BF16 hidden-layer weights, FP32 products; timed like the headline")
         # the same model with the four-body (l = 2) and five-body (l = 1) descriptors added
         mbp = inputs.ModelParams(**{k: getattr(model, k) for k in model.__dataclass_fields__})
         mbp.l_max_4b, mbp.l_max_5b = 2, 1

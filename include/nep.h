@@ -67,12 +67,10 @@ extern "C" {
 #define NEP_FP32 1  /* FP32 descriptors, network and pair forces; FP64 reductions,
                        positions, velocities and integration */
 #define NEP_FP32_BF16 2  /* NEP_FP32 with BF16 hidden-layer weights: W0 (Eq. 2) is rounded
-                            to BF16 once, and both products of the hidden layer (the
-                            pre-activations W0 q and dU/dq = W0^T (w1 (1 - h^2))) run on
-                            tensor cores with each activation split into two BF16 terms
-                            and FP32 accumulation.  The results are the FP32 form's for
-                            the model with BF16-rounded W0, and forces stay the gradient
-                            of its energy. */
+                            to BF16 once, and the hidden layer's products take FP32
+                            activations and accumulate in FP32.  The results are the FP32
+                            form's for the model with BF16-rounded W0, and forces stay the
+                            gradient of its energy. */
 
 /* memory kind of the caller's particle arrays */
 #define NEP_HOST 0

@@ -458,7 +458,7 @@ def nep_set_capacity(h, radial, angular):
 # ---- convenience wrapper -------------------------------------------------------
 class Model:
     """A model handle.  precision: "fp32", "fp64" or "bf16" (FP32 with BF16
-    hidden-layer weights W0 and the hidden layer's products on tensor cores)."""
+    hidden-layer weights W0)."""
 
     def __init__(self, params, precision="fp32", device=0):
         self.params = params

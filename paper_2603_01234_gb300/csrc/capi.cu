@@ -614,7 +614,7 @@ int run_evaluate(nep_model* m, const Plan& p, double* force, double* virial, dou
     a.e = m->e.as<real>();
     a.e_stride = p.Tmax * m->KRP;
     a.phi = m->phi.as<real>();
-    a.net_bf16 = m->precision == NEP_FP32_BF16;
+    a.w0_residual = m->precision == NEP_FP32;
     a.many_body = m->MBT;
     a.perm = m->perm.as<int>();
     a.force = force;
@@ -1668,19 +1668,14 @@ int nep_create(nep_model** out, int n_types, const double* rc_radial, const doub
     // would otherwise add a consistent offset to every site energy)
     o.w0l = o.b0l = o.w1l = o.b1l = o.cRl = -1;
     if (precision != NEP_FP64) {
-        if (T == 1) p = (p + 3) & ~3;
-        o.w0l = p; p += T * hidden * w0s;
+        if (precision == NEP_FP32) {  // BF16 weights W0 have no residual
+            if (T == 1) p = (p + 3) & ~3;
+            o.w0l = p; p += T * hidden * w0s;
+        }
         o.b0l = p; p += T * hidden;
         o.w1l = p; p += T * hidden;
         o.b1l = p; p += T;
         o.cRl = p; p += TT * cRs;
-    }
-    o.w0f = o.w0b = -1;
-    const int nd = m->ND, hp = net_hp(hidden);
-    if (precision == NEP_FP32_BF16) {  // BF16 copies of W0 laid out as MMA B operands
-        p = (p + 3) & ~3;              // 16-byte aligned
-        o.w0f = p; p += T * hp * net_sf(nd) / 2;
-        o.w0b = p; p += T * net_ndp(nd) * (hp + 8) / 2;
     }
     o.total = p;
     std::vector<double> h(p);
@@ -1714,14 +1709,30 @@ int nep_create(nep_model** out, int n_types, const double* rc_radial, const doub
             }
             if (l_max_5b > 0) std::copy(src + k, src + k + m->nA, dst + d3 + m->nA);
         }
+    if (precision == NEP_FP32_BF16) {
+        // W0 rounded to FP32 and then to BF16 (round to nearest even): numbers that FP32
+        // holds exactly, so the form is the FP32 one on another model.  Its two products
+        // ran on tensor cores before, each activation split into two BF16 terms; the
+        // transposes into fragments and the split cost more than the FMAs they replaced
+        for (int k = 0; k < T * hidden * w0s; ++k) {
+            const float f = (float)h[o.w0 + k];
+            uint32_t u;
+            memcpy(&u, &f, 4);
+            if ((u & 0x7fffffffu) > 0x7f800000u) u = 0x7fc00000u;  // NaN
+            else u = (u + 0x7fffu + ((u >> 16) & 1u)) & 0xffff0000u;
+            float r;
+            memcpy(&r, &u, 4);
+            h[o.w0 + k] = (double)r;
+        }
+    }
     std::copy(b0, b0 + T * hidden, h.begin() + o.b0);
     std::copy(w1, w1 + T * hidden, h.begin() + o.w1);
     std::copy(b1, b1 + T, h.begin() + o.b1);
-    if (o.w0l >= 0) {  // rounding residuals of the FP32 tables
+    if (o.b0l >= 0) {  // rounding residuals of the FP32 tables
         auto residual = [&](int hi, int lo, int count) {
             for (int k = 0; k < count; ++k) h[lo + k] = h[hi + k] - (double)(float)h[hi + k];
         };
-        residual(o.w0, o.w0l, T * hidden * w0s);
+        if (o.w0l >= 0) residual(o.w0, o.w0l, T * hidden * w0s);
         residual(o.b0, o.b0l, T * hidden);
         residual(o.w1, o.w1l, T * hidden);
         residual(o.b1, o.b1l, T);
@@ -1738,37 +1749,25 @@ int nep_create(nep_model** out, int n_types, const double* rc_radial, const doub
             return cleanup(fail(NEP_ERR_CUDA, "parameter upload failed"));
     } else {
         std::vector<float> hf(h.begin(), h.end());
-        if (precision == NEP_FP32_BF16) {
-            // W0[t][mu][v] rounded to FP32 and then to BF16 (round to nearest even)
-            auto bf16 = [](double x) -> uint16_t {
-                const float f = (float)x;
-                uint32_t u;
-                memcpy(&u, &f, 4);
-                if ((u & 0x7fffffffu) > 0x7f800000u) return 0x7fc0;  // NaN
-                u += 0x7fffu + ((u >> 16) & 1u);
-                return (uint16_t)(u >> 16);
-            };
-            const int sf = net_sf(nd), ndp = net_ndp(nd), sb = hp + 8;
-            std::vector<uint16_t> wf((size_t)T * hp * sf, 0), wb((size_t)T * ndp * sb, 0);
-            for (int t = 0; t < T; ++t)
-                for (int mu = 0; mu < hidden; ++mu)
-                    for (int v = 0; v < nd; ++v) {
-                        const uint16_t b = bf16(h[o.w0 + ((size_t)t * hidden + mu) * w0s + v]);
-                        wf[((size_t)t * hp + mu) * sf + v] = b;   // [t][mu][v]: X = Q W0^T
-                        wb[((size_t)t * ndp + v) * sb + mu] = b;  // [t][v][mu]: dQ = D W0
-                    }
-            memcpy(hf.data() + o.w0f, wf.data(), wf.size() * 2);
-            memcpy(hf.data() + o.w0b, wb.data(), wb.size() * 2);
-        }
         if (cudaMemcpy(m->params.p, hf.data(), sizeof(float) * p, cudaMemcpyHostToDevice) != cudaSuccess)
             return cleanup(fail(NEP_ERR_CUDA, "parameter upload failed"));
     }
     m->smem_desc = m->real_size * o.total;
-    if (precision == NEP_FP32_BF16)  // plus the per-warp scratch of the network products
-        m->smem_desc = ((m->smem_desc + 15) & ~(size_t)15) + (size_t)(kBlock / 32) * net_scratch(nd);
     // the force kernel stages the cutoff + coefficient prefix only
     m->smem_force = m->real_size * o.n_cut_coef;
-    if (m->smem_desc > 200 * 1024 || m->smem_force > 200 * 1024)
+    // the size limit: what the tables take in shared memory.  The BF16 form's counts W0
+    // three times (two BF16 operand copies beside the rows, and a residual's room) and
+    // the scratch of one block's products, the room its tensor-core version took, so
+    // that the models it takes and refuses stay the same
+    size_t limit = m->smem_desc;
+    if (precision == NEP_FP32_BF16) {
+        const size_t nd = m->ND, hp = (hidden + 15) & ~15, sf = ((nd + 15) & ~(size_t)15) + 8, ndp = (nd + 7) & ~(size_t)7;
+        size_t words = (o.b0l + 3) / 4 * 4 * (T == 1) + (size_t)o.b0l * (T != 1) + (size_t)T * hidden * w0s +
+                       (size_t)(o.total - o.b0l);
+        words = ((words + 3) & ~(size_t)3) + T * hp * sf / 2 + T * ndp * (hp + 8) / 2;
+        limit = ((4 * words + 15) & ~(size_t)15) + (kBlock / 32) * std::max(128 * sf, 128 * (ndp + 1));
+    }
+    if (limit > 200 * 1024 || m->smem_force > 200 * 1024)
         return cleanup(fail(NEP_ERR_ARG, "model too large for shared-memory staging"));
     // the attribute is per kernel, shared by all handles: allow the largest staging size
     const size_t smem_cap = 200 * 1024;
@@ -2370,7 +2369,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     a.e = (real*)(base + L.e);
     a.e_stride = m->T * m->KRP;
     a.phi = (real*)(base + L.phi);
-    a.net_bf16 = m->precision == NEP_FP32_BF16;
+    a.w0_residual = m->precision == NEP_FP32;
     a.many_body = m->MBT;
     a.perm = (int*)(base + L.perm);
     a.force = force ? force : (double*)(base + L.force);

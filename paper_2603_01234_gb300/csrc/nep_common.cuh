@@ -41,20 +41,6 @@ constexpr int kMaxTypes = 16;
 constexpr int kBlock = 128;          // threads per block = particles per work item
 constexpr int kScanItems = 4096;     // cells per block of the scan
 
-// BF16 network tables (the hidden layer as two tensor-core products per warp of
-// 32 particles): padded sizes in BF16 elements.
-__host__ __device__ constexpr int net_kpf(int nd) { return (nd + 15) & ~15; }  // K of X = Q W0^T
-__host__ __device__ constexpr int net_sf(int nd) { return net_kpf(nd) + 8; }    // row stride (bank spread)
-__host__ __device__ constexpr int net_ndp(int nd) { return (nd + 7) & ~7; }     // N of dQ = D W0
-__host__ __device__ constexpr int net_hp(int h) { return (h + 15) & ~15; }       // N of X, K of dQ
-// per-warp shared scratch of the BF16 network, bytes
-__host__ __device__ constexpr int net_scratch(int nd)
-{
-    // two BF16 tiles of Q (head, tail), later one FP32 tile of dQ
-    return (2 * 32 * net_sf(nd) * 2 > 32 * (net_ndp(nd) + 1) * 4 ? 2 * 32 * net_sf(nd) * 2
-                                                                   : 32 * (net_ndp(nd) + 1) * 4);
-}
-
 // Distance (elements) between the type pairs' coefficient tables of n x K entries:
 // odd, so that lanes reading different pairs' tables hit different shared-memory
 // banks.  A compile-time function of the shape, used alike by host and kernels.
@@ -164,10 +150,9 @@ struct ParamLayout {
     int cR, cA;                 // [T][T] tables of [nR][KR] and [nA][KA], coef_stride apart
     int w0, b0, w1, b1;         // [T][H][ND], [T][H], [T][H], [T]
     int w0l, b0l, w1l, b1l;     // FP32 form: the rounding residuals x - (float)x of w0, b0, w1, b1
-                                // (same layouts; -1 in the FP64 form)
+                                // (same layouts; -1 in the FP64 form; w0l -1 with BF16 weights,
+                                // which FP32 holds exactly)
     int cRl;                    // FP32 form: residuals of the cR tables (-1 in the FP64 form)
-    int w0f, w0b;               // BF16-weight network form: W0 as BF16 MMA operands (-1 when absent),
-                                // [T][net_hp(H)][net_sf(ND)] and [T][net_ndp(ND)][net_hp(H) + 8]
     int n_cut_coef;             // elements of the cutoff + coefficient prefix
     int total;                  // all elements
 };
@@ -258,7 +243,7 @@ struct EvalArgs {
     int e_stride;               // Tmax * KRP
     real* phi;                  // FP64 form: [kPsiComp][n][phi_pad(NA)] the sphere-reduced coefficients of
                                 // P_n = sum_lm (dU/dA_nlm) Y_lm, zero padded
-    int net_bf16;               // 1: the hidden layer's products in BF16 on tensor cores
+    int w0_residual;            // 1: W0 has a table of FP32 rounding residuals (the FP32 form)
     int many_body;              // 1: the four- and five-body descriptors follow the three-body ones
     const int* perm;            // sorted slot -> caller index
     double* force;              // per request [3][n_r] blocks (required)
