@@ -224,11 +224,12 @@ struct nep_model {
     int md_n = -1;
     CellGrid md_grid{};
     // workspace
-    Buf cell_of, rec_user, perm_tmp, perm, rec_s, cell_s, cntR, cntA, nlR, nlA, U, e, phi;
+    Buf cell_of, rec_user, perm_tmp, perm, rec_s, cell_s, cntR, cntA, nlR, nlA, U, e;
+    Buf fang;  // FP64 form: each angular pair's force by list slot
     Buf rec32;  // FP64 form: FP32 copies of the sorted records (neighbour screening)
     Buf cell_count, cell_local, block_off, cell_fill, cell_start;
     Buf partial, partial2, counters, gcounters, totals, flags, thermo, sample_index;
-    Buf acc;  // FP32 form: force and virial fixed-point lines, thread virial sums (acc_bytes)
+    Buf acc;  // FP32: force and virial fixed-point lines; virial sums for the totals (acc_bytes)
     bool eval_per_bead = false;  // the evaluation in progress returns per-particle virials
     bool cells_dirty = true;     // the cell counters may be non-zero (a build that failed)
     Buf types_d, pos_d, vel_d, force_d, virial_d, site_d, force_tmp, totals_tmp;
@@ -412,12 +413,16 @@ int single_plan(nep_model* m, int n, const CellGrid& g)
 }
 
 // ---- workspace ---------------------------------------------------------------
-// The FP32 form's accumulators for n particles in one buffer: force lines, virial
-// lines, thread virial sums.
-size_t acc_bytes(size_t n) { return 32 * n + 96 * n + 36 * n; }
+// The accumulators of n particles in one buffer: the FP32 form's force lines and virial
+// lines, then each particle's virial sum (real of rs bytes).
+constexpr size_t acc_bytes(size_t n, size_t rs) { return (rs == 4 ? 128 : 0) * n + 9 * rs * n; }
 unsigned long long* acc_force(void* base) { return (unsigned long long*)base; }
 unsigned long long* acc_virial(void* base, size_t n) { return (unsigned long long*)((char*)base + 32 * n); }
-float* acc_wsum(void* base, size_t n) { return (float*)((char*)base + 128 * n); }
+template <typename real>
+real* acc_wsum(void* base, size_t n)
+{
+    return (real*)((char*)base + (sizeof(real) == 4 ? 128 * n : 0));
+}
 
 int ensure_particles(nep_model* m, int n, int n_items, int n_req, int Tmax)
 {
@@ -433,11 +438,9 @@ int ensure_particles(nep_model* m, int n, int n_items, int n_req, int Tmax)
     NEP_TRY(m->cntA.ensure(sizeof(int) * n));
     NEP_TRY(m->U.ensure(rs * n));
     NEP_TRY(m->e.ensure(rs * Tmax * m->KRP * (size_t)n));
-    if (m->precision == NEP_FP64) NEP_TRY(m->phi.ensure(rs * kPsiComp * phi_pad(m->nA) * (size_t)n));  // FP32 keeps them in registers
     if (m->precision == NEP_FP64) NEP_TRY(m->rec32.ensure(16 * (size_t)n));
     NEP_TRY(m->partial.ensure(sizeof(double) * 10 * (size_t)n_items));
-    // FP32 form: force lines [n][4] u64, virial lines [n][12] u64, thread virial sums [9][n] float
-    if (m->precision != NEP_FP64) NEP_TRY(m->acc.ensure(acc_bytes(n)));
+    NEP_TRY(m->acc.ensure(acc_bytes(n, rs)));
     NEP_TRY(m->partial2.ensure(sizeof(double) * 6 * ((n + kBlock - 1) / kBlock)));
     NEP_TRY(m->force_tmp.ensure(sizeof(double) * 3 * (size_t)n));
     const size_t old_req = m->counters.cap / sizeof(unsigned int);
@@ -446,7 +449,7 @@ int ensure_particles(nep_model* m, int n, int n_items, int n_req, int Tmax)
         NEP_CUDA(cudaMemsetAsync(m->counters.p, 0, m->counters.cap, m->cur));
     NEP_TRY(m->totals.ensure(sizeof(double) * 10 * (size_t)n_req));
     const size_t old_items = m->gcounters.cap;
-    NEP_TRY(m->gcounters.ensure(sizeof(unsigned int) * (size_t)n_items));
+    NEP_TRY(m->gcounters.ensure(2 * sizeof(unsigned int) * (size_t)n_items));  // item groups, then items
     if (m->gcounters.cap != old_items) NEP_CUDA(cudaMemsetAsync(m->gcounters.p, 0, m->gcounters.cap, m->cur));
     return NEP_OK;
 }
@@ -455,6 +458,7 @@ int ensure_lists(nep_model* m, int n)
 {
     NEP_TRY(m->nlR.ensure(sizeof(uint32_t) * (size_t)m->mnR * n));
     NEP_TRY(m->nlA.ensure(sizeof(uint32_t) * (size_t)m->mnA * n));
+    if (m->precision == NEP_FP64) NEP_TRY(m->fang.ensure(3 * sizeof(double) * (size_t)m->mnA * n));
     m->n_lists = n;
     return NEP_OK;
 }
@@ -613,7 +617,7 @@ int run_evaluate(nep_model* m, const Plan& p, double* force, double* virial, dou
     a.U = m->U.as<real>();
     a.e = m->e.as<real>();
     a.e_stride = p.Tmax * m->KRP;
-    a.phi = m->phi.as<real>();
+    a.fang = m->precision == NEP_FP64 ? m->fang.as<real>() : nullptr;
     a.w0_residual = m->precision == NEP_FP32;
     a.many_body = m->MBT;
     a.perm = m->perm.as<int>();
@@ -622,10 +626,11 @@ int run_evaluate(nep_model* m, const Plan& p, double* force, double* virial, dou
     a.site = site;
     a.accF = acc_force(m->acc.p);
     a.accW = acc_virial(m->acc.p, p.n_cap);
-    a.wsum = acc_wsum(m->acc.p, p.n_cap);
+    a.wsum = acc_wsum<real>(m->acc.p, p.n_cap);
     a.partial = m->partial.as<double>();
     a.counter = m->counters.as<unsigned int>() + 2;
     a.gcounter = m->gcounters.as<unsigned int>();
+    a.icounter = a.gcounter + p.items_cap;
     a.err = m->flags.as<int>() + 2;
     a.totals = totals;
     if (kick) {
@@ -705,7 +710,7 @@ int eval_pipeline(nep_model* m, const Plan& p, const int* types_d, const double*
 void put_workspace_ptrs(std::vector<unsigned char>& key, const nep_model* m)
 {
     const Buf* bufs[] = {&m->cell_of, &m->rec_user, &m->perm_tmp, &m->perm, &m->rec_s, &m->cell_s, &m->cntR,
-                         &m->cntA, &m->nlR, &m->nlA, &m->U, &m->e, &m->phi, &m->rec32, &m->cell_count, &m->cell_local,
+                         &m->cntA, &m->nlR, &m->nlA, &m->U, &m->e, &m->fang, &m->rec32, &m->cell_count, &m->cell_local,
                          &m->block_off, &m->cell_fill, &m->cell_start, &m->partial, &m->partial2, &m->counters,
                          &m->gcounters, &m->totals, &m->flags, &m->thermo, &m->sample_index, &m->acc, &m->bussi,
                          &m->md_virial, &m->md_site, &m->heat, &m->heat_rows};
@@ -942,7 +947,7 @@ struct TuneEvents {
 template <typename real>
 int autotune_plan(nep_model* m, const Plan& p, double* force_d)
 {
-    if (m->precision == NEP_FP64) return NEP_OK;  // one FP64 variant only
+    if (evaluate_by_groups(p.items_cap, m->precision == NEP_FP64)) return NEP_OK;  // no variants
     TuneEvents ev;
     for (cudaEvent_t& x : ev.e) NEP_CUDA(cudaEventCreate(&x));
     cudaEvent_t e0 = ev.e[0], em = ev.e[1], e1 = ev.e[2];
@@ -1563,7 +1568,7 @@ int nep_destroy(nep_model* m)
     m->eval_graphs.clear();
     m->timer.destroy();
     Buf* bufs[] = {&m->params, &m->cell_of, &m->rec_user, &m->perm_tmp, &m->perm, &m->rec_s, &m->cell_s, &m->cntR,
-                   &m->cntA, &m->nlR, &m->nlA, &m->U, &m->e, &m->phi, &m->rec32, &m->cell_count, &m->cell_local, &m->block_off,
+                   &m->cntA, &m->nlR, &m->nlA, &m->U, &m->e, &m->fang, &m->rec32, &m->cell_count, &m->cell_local, &m->block_off,
                    &m->cell_fill, &m->cell_start, &m->partial, &m->partial2, &m->counters, &m->gcounters,
                    &m->totals, &m->flags,
                    &m->thermo, &m->sample_index, &m->types_d, &m->pos_d, &m->vel_d, &m->force_d, &m->virial_d,
@@ -1678,6 +1683,17 @@ int nep_create(nep_model** out, int n_types, const double* rc_radial, const doub
         o.cRl = p; p += TT * cRs;
     }
     o.total = p;
+    // the group kernels read W0 and its residuals as 16-byte vectors in every model
+    const int ndv = (m->ND + 3) & ~3;
+    o.w0g = o.w0;
+    o.w0lg = o.w0l;
+    if (T > 1) {
+        p = (p + 3) & ~3;
+        o.w0g = p; p += T * hidden * ndv;
+        if (o.w0l >= 0) {
+            o.w0lg = p; p += T * hidden * ndv;
+        }
+    }
     std::vector<double> h(p);
     for (int k = 0; k < TT; ++k) {
         h[o.rcR2 + k] = m->rcR[k] * m->rcR[k];
@@ -1738,6 +1754,12 @@ int nep_create(nep_model** out, int n_types, const double* rc_radial, const doub
         residual(o.b1, o.b1l, T);
         residual(o.cR, o.cRl, TT * cRs);
     }
+    if (T > 1)
+        for (int k = 0; k < T * hidden; ++k)
+            for (int v = 0; v < m->ND; ++v) {
+                h[o.w0g + (size_t)k * ndv + v] = h[o.w0 + (size_t)k * w0s + v];
+                if (o.w0l >= 0) h[o.w0lg + (size_t)k * ndv + v] = h[o.w0l + (size_t)k * w0s + v];
+            }
 
     auto cleanup = [&](int code) {
         nep_destroy(m);
@@ -2118,13 +2140,13 @@ int nep_request_workspace(nep_model* const* models, int n_models, int model, int
     const size_t rs = m->real_size;
     // cell_of, rec_user, perm_tmp, perm, rec_s, cell_s, cntR, cntA, U, e, force_tmp, partial2
     size_t per_particle = 4 + 4 * rs + 4 + 4 + 4 * rs + 4 + 4 + 4 + rs + rs * Tmax * m->KRP + 24 + 1;
-    if (m->precision == NEP_FP64) per_particle += rs * kPsiComp * phi_pad(m->nA) + 16;
-    else per_particle += acc_bytes(1);            // fixed-point lines, thread virial sums
+    if (m->precision == NEP_FP64) per_particle += 3 * sizeof(double) * (size_t)mnA + 16;  // pair forces, rec32
+    per_particle += acc_bytes(1, rs);             // fixed-point lines, virial sums
     per_particle += 4 * (size_t)(mnR + mnA);      // neighbour lists
     per_particle += 4 + 24 + 24 + 72 + 8;          // host-call staging: types, positions, F, W, U
     const size_t per_cell = 16;                    // count, local prefix, fill, start
     const size_t items = ((size_t)n + kBlock - 1) / kBlock;
-    const size_t per_item = 10 * sizeof(double) + sizeof(WorkItem) + sizeof(unsigned int);  // + group counter
+    const size_t per_item = 10 * sizeof(double) + sizeof(WorkItem) + 2 * sizeof(unsigned int);  // + counters
     const size_t per_req = sizeof(ReqInfo) + 10 * sizeof(double) + sizeof(unsigned int);
     *bytes = per_particle * n + per_cell * g.ncell + per_item * items + per_req;
     return NEP_OK;
@@ -2134,7 +2156,7 @@ int nep_workspace_bytes(nep_model* m, size_t* bytes)
 {
     if (!m || !bytes) return fail(NEP_ERR_ARG, "bad argument");
     const Buf* bufs[] = {&m->cell_of, &m->rec_user, &m->perm_tmp, &m->perm, &m->rec_s, &m->cell_s, &m->cntR,
-                         &m->cntA, &m->nlR, &m->nlA, &m->U, &m->e, &m->phi, &m->rec32, &m->cell_count, &m->cell_local,
+                         &m->cntA, &m->nlR, &m->nlA, &m->U, &m->e, &m->fang, &m->rec32, &m->cell_count, &m->cell_local,
                          &m->block_off, &m->cell_fill, &m->cell_start, &m->partial, &m->partial2, &m->counters,
                          &m->gcounters, &m->totals, &m->flags, &m->thermo, &m->sample_index, &m->types_d,
                          &m->pos_d, &m->vel_d, &m->force_d, &m->virial_d, &m->site_d, &m->force_tmp,
@@ -2197,7 +2219,6 @@ constexpr int kStaticMaxN = 4096;        // particles per call
 constexpr int kStaticMaxCells = 32768;   // cells of the call's grid
 constexpr int kStaticMNR = 256;          // radial neighbours per particle
 constexpr int kStaticMNA = 128;          // angular neighbours per particle
-constexpr int kStaticMaxNA = phi_pad(5);  // padded n_A of the compiled shapes
 constexpr int kStaticMaxT = 4;           // particle types of the model
 constexpr int kStaticMaxKRP = 12;        // padded K_R
 constexpr int kStaticMaxItems = (kStaticMaxN + kBlock - 1) / kBlock;
@@ -2213,12 +2234,12 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Byte layout of the scratch for n particles, ncell cells, real of rs bytes.
 struct StaticLayout {
-    size_t cell_of, rec_user, perm_tmp, perm, rec_s, cell_s, cntR, cntA, U, e, phi, force;
+    size_t cell_of, rec_user, perm_tmp, perm, rec_s, cell_s, cntR, cntA, U, e, fang, force;
     size_t nlR, nlA, cell_count, cell_local, block_off, cell_fill, cell_start;
     size_t partial, counters, totals, flags, tables, acc, end;
 };
 
-constexpr StaticLayout static_layout(size_t n, size_t ncell, size_t rs, size_t nA, size_t ekrp)
+constexpr StaticLayout static_layout(size_t n, size_t ncell, size_t rs, size_t ekrp)
 {
     StaticLayout L{};
     size_t p = 0;
@@ -2232,7 +2253,7 @@ constexpr StaticLayout static_layout(size_t n, size_t ncell, size_t rs, size_t n
     L.cntA = p; p = align256(p + 4 * n);
     L.U = p; p = align256(p + rs * n);
     L.e = p; p = align256(p + rs * ekrp * n);
-    L.phi = p; p = align256(p + rs * kPsiComp * nA * n);
+    L.fang = p; p = align256(p + (rs == 8 ? 3 * rs * (size_t)kStaticMNA * n : 0));  // FP64: pair forces
     L.force = p; p = align256(p + 8 * 3 * n);
     L.nlR = p; p = align256(p + 4 * (size_t)kStaticMNR * n);
     L.nlA = p; p = align256(p + 4 * (size_t)kStaticMNA * n);
@@ -2242,18 +2263,18 @@ constexpr StaticLayout static_layout(size_t n, size_t ncell, size_t rs, size_t n
     L.cell_fill = p; p = align256(p + 4 * ncell);
     L.cell_start = p; p = align256(p + 4 * (ncell + 1));
     L.partial = p; p = align256(p + 8 * 10 * ((n + kBlock - 1) / kBlock));
-    L.counters = p; p = align256(p + 16);
+    L.counters = p; p = align256(p + 16 + 4 * (size_t)kStaticMaxItems);
     L.totals = p; p = align256(p + 8 * 10);
     L.flags = p; p = align256(p + 16);
     L.tables = p; p = align256(p + kStaticTableBytes);
-    L.acc = p; p = align256(p + (rs == 4 ? (32 + 96 + 36) * n : 0));  // FP32 force / virial lines, virial sums
+    L.acc = p; p = align256(p + acc_bytes(n, rs));
     L.end = p;
     return L;
 }
 
-// worst case: FP64, the largest compiled n_A, every limit at its maximum
+// worst case: FP64, every limit at its maximum
 constexpr size_t kStaticScratchBytes =
-    align256(static_layout(kStaticMaxN, kStaticMaxCells, 8, kStaticMaxNA, kStaticMaxT * kStaticMaxKRP).end);
+    align256(static_layout(kStaticMaxN, kStaticMaxCells, 8, kStaticMaxT * kStaticMaxKRP).end);
 
 // The scratch.  In host code this name is only a stand-in for the device symbol;
 // its device address comes from cudaGetSymbolAddress.
@@ -2285,7 +2306,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
 {
     unsigned char* base = nullptr;
     NEP_TRY(static_scratch(m->device, &base));
-    const StaticLayout L = static_layout(n, g.ncell, sizeof(real), phi_pad(m->nA), (size_t)m->T * m->KRP);
+    const StaticLayout L = static_layout(n, g.ncell, sizeof(real), (size_t)m->T * m->KRP);
     if (L.end > kStaticScratchBytes) return fail(NEP_ERR_ARG, "static scratch too small for this call");
     // the request, its work items and the model table, staged through the handle's
     // pinned buffer (allocated by nep_create) into the scratch
@@ -2324,7 +2345,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     // what must start at zero: the overflow/error words and the last-block counter
     // (the cell counters are cleared by the cell build itself)
     NEP_CUDA(cudaMemsetAsync(flags, 0, 16, m->cur));
-    NEP_CUDA(cudaMemsetAsync(counters, 0, 16, m->cur));
+    NEP_CUDA(cudaMemsetAsync(counters, 0, 16 + 4 * (size_t)kStaticMaxItems, m->cur));
     // the scratch's regions move with n, so the cell counters are cleared here
     cudaError_t e = launch_cell_build<real>(
         d_cnt, n, n_items, g.ncell, true, false, d_it, d_rq, d_md, pos, types, (int*)(base + L.cell_of),
@@ -2368,7 +2389,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     a.U = (real*)(base + L.U);
     a.e = (real*)(base + L.e);
     a.e_stride = m->T * m->KRP;
-    a.phi = (real*)(base + L.phi);
+    a.fang = sizeof(real) == 8 ? (real*)(base + L.fang) : nullptr;
     a.w0_residual = m->precision == NEP_FP32;
     a.many_body = m->MBT;
     a.perm = (int*)(base + L.perm);
@@ -2377,10 +2398,11 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     a.site = site_energy;
     a.accF = sizeof(real) == 4 ? acc_force(base + L.acc) : nullptr;
     a.accW = sizeof(real) == 4 ? acc_virial(base + L.acc, n) : nullptr;
-    a.wsum = sizeof(real) == 4 ? acc_wsum(base + L.acc, n) : nullptr;
+    a.wsum = acc_wsum<real>(base + L.acc, n);
     a.partial = (double*)(base + L.partial);
     a.counter = counters;
     a.gcounter = counters + 1;  // one group: at most kStaticMaxN / 128 <= 32 work items
+    a.icounter = counters + 4;
     a.err = flags + 2;
     a.totals = totals;
     e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, n_items, m->smem_desc, m->smem_force, m->cur, nullptr,

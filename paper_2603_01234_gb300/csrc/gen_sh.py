@@ -147,12 +147,13 @@ def emit_reduced():
     for j, (a, b) in enumerate(RED_A + RED_B):
         blk = 0 if j < len(RED_A) else 1
         jj = j if blk == 0 else j - len(RED_A)
-        terms = []
+        term = ""  # explicit multiply-adds: every kernel that inlines this rounds alike
         for i, (ca, cb) in enumerate(cols):
             cf = (ca if blk == 0 else cb)[jj]
             if cf != 0:
-                terms.append(f"real({sp.N(cf, 17)}) * phi[{i}]")
-        out.append(f"    psi[{j}] = {' + '.join(terms) if terms else 'real(0)'};")
+                c = f"real({sp.N(cf, 17)})"
+                term = f"fma({c}, phi[{i}], {term})" if term else f"{c} * phi[{i}]"
+        out.append(f"    psi[{j}] = {term or 'real(0)'};")
     out.append("}")
     return "\n".join(out) + "\n"
 

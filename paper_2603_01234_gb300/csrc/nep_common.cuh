@@ -46,12 +46,8 @@ constexpr int kScanItems = 4096;     // cells per block of the scan
 // banks.  A compile-time function of the shape, used alike by host and kernels.
 __host__ __device__ constexpr int coef_stride(int n, int k) { return (n * k) | 1; }
 
-// Row length of Phi_i per harmonic component: n_A padded to a multiple of 4 so that
-// every row starts on a 16-byte boundary (vector loads).
-__host__ __device__ constexpr int phi_pad(int nA) { return (nA + 3) & ~3; }
-// Coefficients per n of the sphere-reduced form of sum_k dU/dA_nk Y_k, the FP64 form's
-// per-particle angular adjoint (the kShRed of sh_poly.cuh)
-constexpr int kPsiComp = 25;
+// Lanes per particle of the group kernels (evaluate_group.cu).
+constexpr int kGroupLanes = 8;
 
 __host__ __device__ inline uint32_t pack_entry(int j, int dx, int dy, int dz)
 {
@@ -154,7 +150,10 @@ struct ParamLayout {
                                 // which FP32 holds exactly)
     int cRl;                    // FP32 form: residuals of the cR tables (-1 in the FP64 form)
     int n_cut_coef;             // elements of the cutoff + coefficient prefix
-    int total;                  // all elements
+    int total;                  // all elements that a block of the thread-per-particle kernels stages
+    int w0g, w0lg;              // W0 and its residuals in rows padded to a multiple of 4 (vector loads of
+                                // the group kernels): w0 and w0l themselves for one type, else copies
+                                // beyond total
 };
 
 // One model of a batch (device table).
@@ -241,8 +240,7 @@ struct EvalArgs {
     real* U;                    // [n] sorted site energies
     real* e;                    // [n][e_stride] radial gradient folded into the basis
     int e_stride;               // Tmax * KRP
-    real* phi;                  // FP64 form: [kPsiComp][n][phi_pad(NA)] the sphere-reduced coefficients of
-                                // P_n = sum_lm (dU/dA_nlm) Y_lm, zero padded
+    real* fang;                 // FP64 form: [mnA][n][3] each angular pair's f_ij by list slot
     int w0_residual;            // 1: W0 has a table of FP32 rounding residuals (the FP32 form)
     int many_body;              // 1: the four- and five-body descriptors follow the three-body ones
     const int* perm;            // sorted slot -> caller index
@@ -253,11 +251,13 @@ struct EvalArgs {
                                 // left zero by the radial/output kernel
     unsigned long long* accW;   // FP32 form with per-particle virials: [n][12] fixed-point W[9] (2^-32 eV),
                                 // same rules; used only when virial is non-null
-    float* wsum;                // FP32 form: [9][n] each thread's angular virial sum (for the totals)
+    real* wsum;                 // [9][n] each particle's virial sum for the totals (FP32: its angular part
+                                // until the force kernel adds the radial part)
     double* partial;            // [items][10] per work item (E, W[9])
     unsigned int* counter;      // [requests] last-group counters (self-resetting)
     unsigned int* gcounter;     // [items] last-block counters of the item groups, at each
                                 // group's first item (self-resetting)
+    unsigned int* icounter;     // [items] group kernels: finished blocks of each item (self-resetting)
     double* totals;             // [requests][10]: E, W[9]
     int* err = nullptr;         // the error word (kErrCellList on an inconsistent cell list)
     // MD: the step's closing half-kick applied by the output pass as soon as F_i is
@@ -300,13 +300,21 @@ template <typename real>
 cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, size_t smem, cudaStream_t st);
 
 // Shape-dispatched evaluation; returns cudaErrorInvalidValue for an uncompiled shape.
-// mb_desc / mb_force: resident blocks per SM of the FP32 kernel variants (2 or 3; the
-// force kernel also 4).  The FP64 form has one effective variant of each.
-// The FP32 form needs a.acc (the scatter accumulators); the FP64 form ignores it.
+// mb_desc / mb_force / ch_force: the variants of the thread-per-particle kernels
+// (resident blocks per SM, walk chunk), which evaluate_by_groups says are not used.
 template <typename real>
 cudaError_t launch_evaluate(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap, size_t smem_desc,
                             size_t smem_force, cudaStream_t st, cudaEvent_t mid = nullptr, int mb_desc = 3,
                             int mb_force = 3, int ch_force = 4);
+
+// Whether a batch of items_cap work items runs the group kernels (which have no variants).
+bool evaluate_by_groups(int items_cap, bool fp64);
+
+template <typename real>
+cudaError_t launch_evaluate_group(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap,
+                                  cudaStream_t st, cudaEvent_t mid);
+template <typename real>
+cudaError_t group_set_smem();
 
 template <typename real>
 bool evaluate_shape_supported(int nR, int nA, int KR, int KA);
