@@ -1712,6 +1712,14 @@ int nep_create(nep_model** out, int n_types, const double* rc_radial, const doub
         std::copy(c_angular + (size_t)k * m->nA * m->KA, c_angular + (size_t)(k + 1) * m->nA * m->KA,
                   h.begin() + o.cA + k * cAs);
     }
+    // column 0 of the angular tables as the kernels use it (cheb_sum): 2 c_0 + sum_{k>=1} c_k
+    for (int k = 0; k < TT; ++k)
+        for (int nn = 0; nn < m->nA; ++nn) {
+            double* row = h.data() + o.cA + (size_t)k * cAs + (size_t)nn * m->KA;
+            double s = row[0];
+            for (int q = 0; q < m->KA; ++q) s += row[q];
+            row[0] = s;
+        }
     for (int t = 0; t < T; ++t)
         for (int mu = 0; mu < hidden; ++mu) {
             const double* src = w0 + ((size_t)t * hidden + mu) * nd_user;

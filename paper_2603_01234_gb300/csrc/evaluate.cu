@@ -169,8 +169,8 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
         const real inv_r = rsqrt_r(r2);
         const real r = r2 * inv_r;
         const int tp = ti * T + rj.t;
-        real f[KA];
-        basis<real, KA>(r, P[off.rcAi + tp], P[off.rcAl + tp], f);
+        real hf, t[KA];
+        cheb_T<real, KA>(r, P[off.rcAi + tp], P[off.rcAl + tp], hf, t);
         real Y[kNLM];
         sh_eval(dx * inv_r, dy * inv_r, dz * inv_r, Y);
         const real* crow = P + off.cA + tp * coef_stride(NA, KA);
@@ -180,9 +180,7 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
             // every row up front, which would hold 32 more registers across the sums
             real cr[KA];
             load_coef(crow + nn * KA, T == 1 && KA % 4 == 0, cr);
-            real g = real(0);
-#pragma unroll
-            for (int k = 0; k < KA; ++k) g += cr[k] * f[k];
+            const real g = hf * cheb_sum(cr, t);
 #pragma unroll
             for (int k = 0; k < kNLM; ++k) A[nn][k] += g * Y[k];
             asm volatile("" ::: "memory");
@@ -427,22 +425,15 @@ __device__ __forceinline__ void force_angular_phi_reg(const EvalArgs<real>& a, c
         const real inv_r = rsqrt_r(r2);
         const real r = r2 * inv_r;
         const int tij = ti * T + rj.t;
-        real f[KA], df[KA];
-        basis_d<real, KA>(r, P[off.rcAi + tij], P[off.rcAl + tij], f, df);
+        real hf, hdf, hdx, t[KA], dt[KA];
+        cheb_dT<real, KA>(r, P[off.rcAi + tij], P[off.rcAl + tij], hf, hdf, hdx, t, dt);
         real g[NA], dg[NA];
         const real* crow = P + off.cA + tij * coef_stride(NA, KA);
 #pragma unroll
         for (int nn = 0; nn < NA; ++nn) {
             real cr[KA];  // one row at a time (see the angular moments)
             load_coef(crow + nn * KA, T == 1 && KA % 4 == 0, cr);
-            real s0 = real(0), s1 = real(0);
-#pragma unroll
-            for (int k = 0; k < KA; ++k) {
-                s0 += cr[k] * f[k];
-                s1 += cr[k] * df[k];
-            }
-            g[nn] = s0;
-            dg[nn] = s1;
+            cheb_g_dg(cr, t, dt, hf, hdf, hdx, g[nn], dg[nn]);
             asm volatile("" ::: "memory");
         }
         const real ux = dx * inv_r, uy = dy * inv_r, uz = dz * inv_r;

@@ -211,17 +211,14 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
             if (ok) {
                 const Pair<real> p = make_pair(ri, rc, ec, len);
                 const int tp = ti * T + p.tj;
-                real f[KA];
-                basis<real, KA>(p.r, P[off.rcAi + tp], P[off.rcAl + tp], f);
+                real hf, t[KA];
+                cheb_T<real, KA>(p.r, P[off.rcAi + tp], P[off.rcAl + tp], hf, t);
                 const real* crow = P + off.cA + tp * coef_stride(NA, KA);
 #pragma unroll
                 for (int nn = 0; nn < NA; ++nn) {
                     real cr[KA];
                     load_coef(crow + nn * KA, T == 1 && KA % 4 == 0, cr);
-                    real s = real(0);
-#pragma unroll
-                    for (int k = 0; k < KA; ++k) s = fma(cr[k], f[k], s);
-                    g[nn] = s;
+                    g[nn] = hf * cheb_sum(cr, t);
                 }
                 sh_eval(p.dx * p.inv_r, p.dy * p.inv_r, p.dz * p.inv_r, Y);
             } else {  // a zero row adds exact zeros
@@ -422,8 +419,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
         if (s < cA) {
             const Pair<real> p = make_pair(ri, rc, ec, len);
             const int tij = ti * T + p.tj;
-            real f[KA], df[KA];
-            basis_d<real, KA>(p.r, P[off.rcAi + tij], P[off.rcAl + tij], f, df);
+            real hf, hdf, hdx, t[KA], dt[KA];
+            cheb_dT<real, KA>(p.r, P[off.rcAi + tij], P[off.rcAl + tij], hf, hdf, hdx, t, dt);
             const real* crow = P + off.cA + tij * coef_stride(NA, KA);
             const real ux = p.dx * p.inv_r, uy = p.dy * p.inv_r, uz = p.dz * p.inv_r;
             real D = real(0);
@@ -432,12 +429,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
             for (int nn = 0; nn < NA; ++nn) {
                 real cr[KA];
                 load_coef(crow + nn * KA, T == 1 && KA % 4 == 0, cr);
-                real g = real(0), dg = real(0);
-#pragma unroll
-                for (int k = 0; k < KA; ++k) {
-                    g = fma(cr[k], f[k], g);
-                    dg = fma(cr[k], df[k], dg);
-                }
+                real g, dg;
+                cheb_g_dg(cr, t, dt, hf, hdf, hdx, g, dg);
                 real c[GT::PSI];
                 loadN<real, GT::PSI>(psi + nn * GT::PSI, c);
                 real v, vx, vy, vz;

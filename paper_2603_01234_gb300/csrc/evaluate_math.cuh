@@ -93,6 +93,66 @@ __device__ __forceinline__ void basis_acc(real r, real inv_rc, real inv_lo, real
     }
 }
 
+// The angular functions g_n(r) = sum_k c_nk f_k(r) are evaluated from the Chebyshev sums:
+//   g_n = (f_c/2) P_n(x),  P_n = c'_n0 + sum_{k>=1} c_nk T_k(x),  c'_n0 = 2 c_n0 + sum_{k>=1} c_nk,
+//   g_n' = (f_c/2) x' sum_{k>=1} c_nk T_k'(x) + (f_c'/2) P_n,
+// with c' in place of c in column 0 of the angular tables, so the f_k and f_k' themselves
+// need not be formed.  cheb_T: f_c/2 and T_k; cheb_dT: f_c/2, f_c'/2, x' f_c/2, T_k, T_k'
+// (entry 0 unused).
+template <typename real, int K>
+__device__ __forceinline__ void cheb_T(real r, real inv_rc, real inv_lo, real& hf, real (&t)[K])
+{
+    const real xr = scaled_r(r, inv_rc, inv_lo);
+    hf = cut_half(xr);
+    const real s = xr - real(1);
+    const real x = fma(real(2) * s, s, real(-1));
+    const real x2 = x + x;
+    t[0] = real(1);
+    t[1] = x;
+#pragma unroll
+    for (int k = 2; k < K; ++k) t[k] = fma(x2, t[k - 1], -t[k - 2]);
+}
+template <typename real, int K>
+__device__ __forceinline__ void cheb_dT(real r, real inv_rc, real inv_lo, real& hf, real& hdf, real& hdx, real (&t)[K],
+                                        real (&d)[K])
+{
+    const real xr = scaled_r(r, inv_rc, inv_lo);
+    cut_half_d(xr, inv_rc, &hf, &hdf);
+    const real s = xr - real(1);
+    const real x = fma(real(2) * s, s, real(-1));
+    hdx = real(4) * s * inv_rc * hf;
+    const real x2 = x + x;
+    t[0] = real(1);
+    t[1] = x;
+    d[0] = real(0);
+    d[1] = real(1);
+#pragma unroll
+    for (int k = 2; k < K; ++k) {  // T'_k = 2 T_{k-1} + 2 x T'_{k-1} - T'_{k-2}
+        t[k] = fma(x2, t[k - 1], -t[k - 2]);
+        d[k] = fma(real(2), t[k - 1], fma(x2, d[k - 1], -d[k - 2]));
+    }
+}
+template <typename real, int K>
+__device__ __forceinline__ real cheb_sum(const real (&c)[K], const real (&t)[K])
+{
+    real p = c[0];
+#pragma unroll
+    for (int k = 1; k < K; ++k) p = fma(c[k], t[k], p);
+    return p;
+}
+// g_n and g_n' from one row of coefficients
+template <typename real, int K>
+__device__ __forceinline__ void cheb_g_dg(const real (&c)[K], const real (&t)[K], const real (&d)[K], real hf, real hdf,
+                                          real hdx, real& g, real& dg)
+{
+    const real p = cheb_sum(c, t);
+    real q = c[1];
+#pragma unroll
+    for (int k = 2; k < K; ++k) q = fma(c[k], d[k], q);
+    g = hf * p;
+    dg = fma(hdx, q, hdf * p);
+}
+
 // f_k and df_k/dr:  df_k = 1/2 [T_k'(x) x'(r) f_c + (T_k + 1) f_c'],
 // with T'_{k+1} = 2 T_k + 2 x T'_k - T'_{k-1}.
 template <typename real, int K>

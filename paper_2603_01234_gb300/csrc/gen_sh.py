@@ -1,6 +1,5 @@
-"""Generate sh_poly.cuh: real orthonormal spherical harmonics l = 1..4 as homogeneous
-harmonic polynomials of the unit vector (the angular moments of Eq. 5), and the
-harmonics' sphere-reduced form (z^2 = 1 - x^2 - y^2) from which the angular pair
+"""Generate sh_poly.cuh: real orthonormal spherical harmonics l = 1..4 of the unit vector
+(the angular moments of Eq. 5), and the harmonics' sphere-reduced form (z^2 = 1 - x^2 - y^2) from which the angular pair
 forces are evaluated.
 
 Run with sympy available:  python gen_sh.py > sh_poly.cuh
@@ -60,33 +59,67 @@ def check():
     assert np.abs((M * w) @ M.T - np.eye(len(KEYS))).max() < 1e-12
 
 
-def c(expr):
-    e = sp.expand(sp.N(expr, 20))
-    s = sp.ccode(e)
-    # numeric literals -> real(...) so that float kernels stay in float
-    import re
-    s = re.sub(r"(\d+\.\d+(e[-+]?\d+)?)", r"real(\1)", s)
-    return re.sub(r"pow\(([xyz]), (\d)\)", r"\1\2", s)
+# The harmonics on the unit sphere.  With x^2 + y^2 + z^2 = 1 each Y_lm factors into a few
+# shared polynomials, about 50 operations for all 24 where the homogeneous forms take 140.
+# Each line assigns one name; the lines are C and Python alike, so check_eval evaluates
+# the very text that is emitted.  Multiply-adds are explicit.
+def N(v):
+    return f"real({sp.N(v, 17)})"
 
 
-MONO = ("    const real x2 = x * x, y2 = y * y, z2 = z * z, x3 = x2 * x, y3 = y2 * y, z3 = z2 * z;\n"
-        "    const real x4 = x2 * x2, y4 = y2 * y2, z4 = z2 * z2;\n"
-        "    (void)x3; (void)y3; (void)z3; (void)x4; (void)y4; (void)z4;")
+def eval_lines():
+    c1 = S(3 / (4 * pi))
+    c2, c20, c22 = S(15 / pi) / 2, S(5 / pi) / 4, S(15 / pi) / 4
+    c33, c32, c32z, c31, c30 = S(35 / (2 * pi)) / 4, S(105 / pi) / 2, S(105 / pi) / 4, S(21 / (2 * pi)) / 4, S(7 / pi) / 4
+    c44, c44x = Q(3, 16) * S(35 / pi), Q(3, 4) * S(35 / pi)
+    c43, c42, c42x = Q(3, 4) * S(35 / (2 * pi)), Q(3, 8) * S(5 / pi), Q(3, 4) * S(5 / pi)
+    c41, c40 = Q(3, 4) * S(5 / (2 * pi)), Q(3, 16) * S(1 / pi)
+    return [
+        ("x2", "x * x"), ("y2", "y * y"), ("z2", "z * z"), ("xy", "x * y"), ("xz", "x * z"), ("yz", "y * z"),
+        ("dd", "fma(x, x, -y2)"),            # x^2 - y^2
+        ("p3", "fma(real(3), x2, -y2)"),     # 3 x^2 - y^2
+        ("m3", "fma(real(-3), y2, x2)"),     # x^2 - 3 y^2
+        ("a3", f"fma({N(5 * c31)}, z2, {N(-c31)})"),      # c31 (5 z^2 - 1)
+        ("t4", f"fma({N(7 * c41)}, z2, {N(-3 * c41)})"),  # c41 (7 z^2 - 3)
+        ("Y[0]", f"{N(c1)} * y"), ("Y[1]", f"{N(c1)} * z"), ("Y[2]", f"{N(c1)} * x"),
+        ("Y[3]", f"{N(c2)} * xy"), ("Y[4]", f"{N(c2)} * yz"), ("Y[5]", f"fma({N(3 * c20)}, z2, {N(-c20)})"),
+        ("Y[6]", f"{N(c2)} * xz"), ("Y[7]", f"{N(c22)} * dd"),
+        ("Y[8]", f"{N(c33)} * y * p3"), ("Y[9]", f"{N(c32)} * xy * z"), ("Y[10]", "y * a3"),
+        ("Y[11]", f"z * fma({N(5 * c30)}, z2, {N(-3 * c30)})"), ("Y[12]", "x * a3"),
+        ("Y[13]", f"{N(c32z)} * z * dd"), ("Y[14]", f"{N(c33)} * x * m3"),
+        ("Y[15]", f"{N(c44x)} * xy * dd"), ("Y[16]", f"{N(c43)} * yz * p3"),
+        ("Y[17]", f"xy * fma({N(7 * c42x)}, z2, {N(-c42x)})"), ("Y[18]", "yz * t4"),
+        ("Y[19]", f"fma(fma({N(35 * c40)}, z2, {N(-30 * c40)}), z2, {N(3 * c40)})"), ("Y[20]", "xz * t4"),
+        ("Y[21]", f"dd * fma({N(7 * c42)}, z2, {N(-c42)})"), ("Y[22]", f"{N(c43)} * xz * m3"),
+        ("Y[23]", f"{N(c44)} * fma(x2, m3, -(y2 * p3))"),
+    ]
+
+
+def check_eval():
+    """The emitted lines equal the harmonics on random points of the sphere."""
+    rng = np.random.default_rng(8)
+    u = rng.standard_normal((3, 400))
+    u /= np.linalg.norm(u, axis=0)
+    env = {"x": u[0], "y": u[1], "z": u[2], "real": float, "fma": lambda p, q, r: p * q + r, "Y": [None] * 24}
+    for name, expr in eval_lines():
+        exec(f"{name} = {expr}", env)
+    for i, k in enumerate(KEYS):
+        want = sp.lambdify((x, y, z), Y[k], "numpy")(*u)
+        assert np.abs(env["Y"][i] - want).max() < 1e-13, k
 
 
 def emit():
     out = []
     out.append("// Generated by gen_sh.py -- real orthonormal spherical harmonics, l = 1..4.")
-    out.append("// Index k = l*l - 1 + (m + l); each Y_k is a homogeneous harmonic polynomial of")
-    out.append("// degree l in the components of the unit vector (x, y, z).")
+    out.append("// Index k = l*l - 1 + (m + l).  (x, y, z) is a unit vector: the forms use")
+    out.append("// x^2 + y^2 + z^2 = 1 and hold on the sphere only.")
     out.append("#pragma once")
     out.append("")
     out.append("template <typename real>")
     out.append("__device__ __forceinline__ void sh_eval(real x, real y, real z, real* Y)")
     out.append("{")
-    out.append(MONO)
-    for i, k in enumerate(KEYS):
-        out.append(f"    Y[{i}] = {c(Y[k])};")
+    for name, expr in eval_lines():
+        out.append(f"    {'' if name.startswith('Y') else 'const real '}{name} = {expr};")
     out.append("}")
     return "\n".join(out) + "\n"
 
@@ -160,6 +193,7 @@ def emit_reduced():
 
 if __name__ == "__main__":
     check()
+    check_eval()
     check_reduced()
     sys.stdout.write(emit())
     sys.stdout.write(emit_reduced())
