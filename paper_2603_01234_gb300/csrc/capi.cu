@@ -558,6 +558,11 @@ int run_kick_drift_cells(nep_model* m, const Plan& p, const int* types_d, const 
     return NEP_OK;
 }
 
+int plan_form(const nep_model* m, const Plan& p)
+{
+    return neighbor_form(p.items_cap, p.n, p.ncell, m->precision == NEP_FP64);
+}
+
 template <typename real>
 int run_neighbors(nep_model* m, const Plan& p)
 {
@@ -584,7 +589,7 @@ int run_neighbors(nep_model* m, const Plan& p)
     a.rec32 = m->precision == NEP_FP64 ? m->rec32.as<PosRec<float>>() : nullptr;
     if ((uint64_t)std::max(a.mnR, a.mnA) * (uint64_t)a.n > (1ull << 32))
         return fail(NEP_ERR_ARG, "neighbour lists beyond 2^32 entries (capacity x particles)");
-    cudaError_t e = launch_neighbors<real>(a, p.items_cap, p.smem_nbr, m->cur);
+    cudaError_t e = launch_neighbors<real>(a, p.items_cap, plan_form(m, p), p.smem_nbr, m->cur);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("neighbours: ") + cudaGetErrorString(e));
     return NEP_OK;
 }
@@ -731,7 +736,8 @@ std::vector<unsigned char> eval_graph_key(const nep_model* m, const Plan& p, con
         key.insert(key.end(), b, b + sz);
     };
     const int ints[] = {p.n_cap, p.items_cap, p.ncell_cap, p.Tmax, m->mnR, m->mnA, m->mb_desc, m->mb_force, m->ch_force,
-                        m->eval_per_bead ? 1 : 0, m->precision, m->MBT, (int)sizeof(real)};
+                        m->eval_per_bead ? 1 : 0, m->precision, m->MBT, (int)sizeof(real),
+                        plan_form(m, p)};
     put(ints, sizeof ints);
     const size_t sm[] = {p.smem_desc, p.smem_force, p.smem_nbr, p.off_reqs, p.off_items, p.off_models};
     put(sm, sizeof sm);
@@ -2379,7 +2385,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     na.maxcnt = flags;
     na.accF = sizeof(real) == 4 ? acc_force(base + L.acc) : nullptr;
     na.accW = sizeof(real) == 4 && virial ? acc_virial(base + L.acc, n) : nullptr;
-    e = launch_neighbors<real>(na, n_items, neighbor_smem<real>(m->T), m->cur);
+    e = launch_neighbors<real>(na, n_items, neighbor_form(n_items, n, g.ncell, sizeof(real) == 8), neighbor_smem<real>(m->T), m->cur);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("neighbours: ") + cudaGetErrorString(e));
     EvalArgs<real> a;
     a.n = n;

@@ -9,7 +9,7 @@
 //                and gather the records into cell order
 //   k_neighbors  one thread per particle scans the (2S+1)^3 surrounding cells and
 //                writes the radial (r < r_c^R) and angular (r < r_c^A) lists
-//                (k_neighbors_warp: one warp per particle, for small batches)
+//                (k_neighbors_warp: warps take one or eight particles, for smaller batches)
 #include "nep_common.cuh"
 
 namespace nep {
@@ -420,7 +420,7 @@ __device__ __forceinline__ void neighbors_item(const NeighborArgs<real>& a, cons
                     }
                     const int cell = q.cell_base + (z * ncy + y) * ncx + x;
                     // j's position relative to i is (r_j + offset) - r_i = r_j - b
-                    const real bx = ri.x - (real)dx * lx, by = ri.y - (real)dy * ly, bz = ri.z - (real)dz * lz;
+                    const real bx = fma(-(real)dx, lx, ri.x), by = fma(-(real)dy, ly, ri.y), bz = fma(-(real)dz, lz, ri.z);
                     const uint32_t code = ((uint32_t)((dx + 2) | ((dy + 2) << 3) | ((dz + 2) << 6))) << kJBits;
                     const int kb = a.cell_start[cell], ke = a.cell_start[cell + 1];  // within [0, n] (k_scatter)
                     // branch-free body: the tests predicate the stores and the counts; i
@@ -428,7 +428,7 @@ __device__ __forceinline__ void neighbors_item(const NeighborArgs<real>& a, cons
                     // for only in i's own cell (center: the same for every lane of the warp)
                     auto candidate = [&](int k, const PosRec<real>& rj, real cR2, real cA2, bool center) {
                         const real ddx = rj.x - bx, ddy = rj.y - by, ddz = rj.z - bz;
-                        const real r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+                        const real r2 = fma(ddz, ddz, fma(ddy, ddy, ddx * ddx));  // as in k_neighbors_warp
                         const uint32_t ent = (uint32_t)k | code;
                         const bool other = !center || k != i;
                         const bool inR = (r2 < cR2) & other, inA = (r2 < cA2) & other;
@@ -451,7 +451,7 @@ __device__ __forceinline__ void neighbors_item(const NeighborArgs<real>& a, cons
                         if (j_far || (r2f < scrR[tp + 1]) != inR || (r2f < scrA[tp + 1]) != inA) {
                             const PosRec<real> rj = ldg_rec(a.rec + k);
                             const real ddx = rj.x - bx, ddy = rj.y - by, ddz = rj.z - bz;
-                            const real r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+                            const real r2 = fma(ddz, ddz, fma(ddy, ddy, ddx * ddx));  // as in k_neighbors_warp
                             inR = r2 < cutR[rf.t];
                             inA = r2 < cutA[rf.t];
                         }
@@ -523,116 +523,257 @@ __device__ __forceinline__ void neighbors_item(const NeighborArgs<real>& a, cons
     }
 }
 
-// Small batches: one warp per particle.  With few work items the thread-per-particle
-// kernel leaves most SMs idle and each thread's candidate loop (about 500 candidates
-// for water) is the whole kernel's latency.  Here the warp's lanes test 32 of the
-// particle's candidates at a time (consecutive records of one stencil cell, a
-// coalesced load), and ballots compact the accepted ones in candidate order, so the
-// lists are exactly those the thread-per-particle kernel writes.  A block of kBlock
-// threads takes kBlock / 32 particles of one work item.
-constexpr int kNbrWarpParticles = kBlock / 32;
+// The warp kernel enumerates a particle's candidates as runs: for each of the
+// (2 S_y + 1)(2 S_z + 1) rows of cells along x around it, the cells x - S_x ... x + S_x are
+// consecutive, and so are their records in sorted order (periodic axes: one run per image
+// of the row).  The lanes look the runs' bounds up side by side and then walk the
+// records of all runs behind one another, 32 at a time and one step ahead with the loads,
+// so that no chain of dependent loads is left between two cells (cell by cell it took
+// 22 us for 512 particles, this way 14).  It applies k_neighbors' distance test in the same
+// order, so both write the same lists.
 
-template <typename real>
-__global__ void __launch_bounds__(kBlock) k_neighbors_warp(NeighborArgs<real> a)
+// Runs of one warp, in list order (dz, dy, x): run r holds the candidates [first[r],
+// first[r + 1]).
+constexpr int kNbrRuns = 32;
+struct NbrRuns {
+    int first[kNbrRuns + 1];
+    int4 run[kNbrRuns];  // record of candidate 0, row's first cell - image shift, dy, dz
+};
+
+// A candidate: its record, and its cell's offset (dx from cell xref).
+struct NbrCand {
+    int k, dx, dy, dz;
+};
+
+// Walks the candidates of a run table 32 at a time; the lane's run moves on with its
+// candidate.
+struct NbrCursor {
+    int r = 0;
+    __device__ __forceinline__ NbrCand at(const NbrRuns& R, int f, const int* cell_s, int xref)
+    {
+        while (f >= R.first[r + 1]) ++r;
+        const int4 v = R.run[r];
+        NbrCand c;
+        c.k = v.x + f;
+        c.dx = cell_s[c.k] - v.y - xref;
+        c.dy = v.z;
+        c.dz = v.w;
+        return c;
+    }
+};
+
+// The runs r0 ... r0 + 31 of the rows of cells around cell (cx, cy, cz); returns the number of
+// their candidates.  A warp calls it as a whole.
+__device__ __forceinline__ int nbr_runs(NbrRuns& R, const CellGrid& g, int cell_base, const int* cell_start, int cx,
+                                        int cy, int cz, int images, int r0, int runs)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    real* cut = reinterpret_cast<real*>(smem_raw);  // rcR2[T*T], rcA2[T*T]
-    constexpr int kPerItem = kBlock / kNbrWarpParticles;  // blocks per work item
-    const int item = (int)blockIdx.x / kPerItem;
-    if (item >= a.counts->n_items) return;
-    const WorkItem it = a.items[item];
-    const ReqInfo& q = a.reqs[it.req];
-    const ModelDesc<real> md = a.models[q.model];
-    const int T = md.T, TT = T * T;
-    for (int k = threadIdx.x; k < TT; k += blockDim.x) {
-        cut[k] = md.params[md.off.rcR2 + k];
-        cut[TT + k] = md.params[md.off.rcA2 + k];
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    const int i = it.begin + ((int)blockIdx.x % kPerItem) * kNbrWarpParticles + ((int)threadIdx.x >> 5);
-    if (i >= it.end) return;  // warp-uniform
-    const CellGrid& g = q.g;
-    const PosRec<real> ri = a.rec[i];
-    const int c = min(max(a.cell_s[i] - q.cell_base, 0), g.ncell - 1);  // clamped as in k_neighbors
-    const int cx = c % g.nc[0], cy = (c / g.nc[0]) % g.nc[1], cz = c / (g.nc[0] * g.nc[1]);
-    const real* cutR = cut + ri.t * T;
-    const real* cutA = cut + TT + ri.t * T;
-    const real lx = (real)g.len[0], ly = (real)g.len[1], lz = (real)g.len[2];
-    const int ncx = g.nc[0], ncy = g.nc[1], ncz = g.nc[2];
-    const uint32_t stride = (uint32_t)a.n, col = (uint32_t)i;
-    int nr = 0, na = 0;  // warp-uniform
-    for (int dz = -g.S[2]; dz <= g.S[2]; ++dz) {
-        int z = cz + dz;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, r = r0 + lane;
+    const int ny = 2 * g.S[1] + 1;
+    int kb = 0, len = 0;
+    int4 v = make_int4(0, 0, 0, 0);
+    if (r < runs) {
+        const int img = r % images, rr = r / images;
+        const int dy = rr % ny - g.S[1], dz = rr / ny - g.S[2];
+        int y = cy + dy, z = cz + dz;
+        bool ok = true;
+        if (g.pbc[1]) {  // |dy| <= 2, so at most two corrections even for one cell per axis
+            while (y < 0) y += g.nc[1];
+            while (y >= g.nc[1]) y -= g.nc[1];
+        } else {
+            ok = y >= 0 && y < g.nc[1];
+        }
         if (g.pbc[2]) {
-            while (z < 0) z += ncz;
-            while (z >= ncz) z -= ncz;
-        } else if (z < 0 || z >= ncz) {
-            continue;
+            while (z < 0) z += g.nc[2];
+            while (z >= g.nc[2]) z -= g.nc[2];
+        } else {
+            ok &= z >= 0 && z < g.nc[2];
         }
-        for (int dy = -g.S[1]; dy <= g.S[1]; ++dy) {
-            int y = cy + dy;
-            if (g.pbc[1]) {
-                while (y < 0) y += ncy;
-                while (y >= ncy) y -= ncy;
-            } else if (y < 0 || y >= ncy) {
-                continue;
-            }
-            for (int dx = -g.S[0]; dx <= g.S[0]; ++dx) {
-                int x = cx + dx;
-                if (g.pbc[0]) {
-                    while (x < 0) x += ncx;
-                    while (x >= ncx) x -= ncx;
-                } else if (x < 0 || x >= ncx) {
-                    continue;
-                }
-                const int cell = q.cell_base + (z * ncy + y) * ncx + x;
-                const real bx = ri.x - (real)dx * lx, by = ri.y - (real)dy * ly, bz = ri.z - (real)dz * lz;
-                const uint32_t code = ((uint32_t)((dx + 2) | ((dy + 2) << 3) | ((dz + 2) << 6))) << kJBits;
-                const int kb = a.cell_start[cell], ke = a.cell_start[cell + 1];  // within [0, n] (k_scatter)
-                const int self = (dx == 0 && dy == 0 && dz == 0) ? i : -1;
-                for (int k0 = kb; k0 < ke; k0 += 32) {
-                    const int k = k0 + lane;
-                    bool inR = false, inA = false;
-                    if (k < ke) {
-                        const PosRec<real> rj = ldg_rec(a.rec + k);
-                        const real ddx = rj.x - bx, ddy = rj.y - by, ddz = rj.z - bz;
-                        const real r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-                        const bool other = k != self;
-                        inR = (r2 < cutR[rj.t]) & other;
-                        inA = (r2 < cutA[rj.t]) & other;
-                    }
-                    const unsigned mR = __ballot_sync(0xffffffffu, inR), mA = __ballot_sync(0xffffffffu, inA);
-                    const uint32_t ent = (uint32_t)k | code;
-                    const int sR = nr + __popc(mR & below), sA = na + __popc(mA & below);
-                    if (inR && sR < a.mnR) a.nlR[(uint32_t)sR * stride + col] = ent;
-                    if (inA && sA < a.mnA) a.nlA[(uint32_t)sA * stride + col] = ent;
-                    nr += __popc(mR);
-                    na += __popc(mA);
-                }
-            }
+        // the images of the row that cx - S_x ... cx + S_x touches, the first one holding its start
+        const int ncx = g.nc[0];
+        int x0 = cx - g.S[0], x1 = cx + g.S[0], shift = 0;
+        if (g.pbc[0]) {
+            int w = 0;
+            for (int x = x0; x < 0; x += ncx) --w;
+            shift = (w + img) * ncx;
+        }
+        x0 = max(x0 - shift, 0);
+        x1 = min(x1 - shift, ncx - 1);
+        if (ok && x0 <= x1) {
+            const int base = cell_base + (z * g.nc[1] + y) * ncx;
+            kb = cell_start[base + x0];
+            len = max(cell_start[base + x1 + 1] - kb, 0);  // both within [0, n] (k_scatter)
+            v = make_int4(0, base - shift, dy, dz);
         }
     }
-    if (lane == 0) {
-        a.cntR[i] = nr;
-        a.cntA[i] = na;
-        atomicMax(&a.maxcnt[0], nr);
-        atomicMax(&a.maxcnt[1], na);
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, incl, o);
+        if (lane >= o) incl += y;
     }
-    if (a.accF && lane < 2) {  // i's fixed-point lines start the evaluation at zero
-        reinterpret_cast<ulonglong2*>(a.accF + (size_t)i * 4)[lane] = make_ulonglong2(0ull, 0ull);
+    v.x = kb - (incl - len);
+    __syncwarp();
+    if (lane == 0) R.first[0] = 0;
+    R.first[lane + 1] = incl;
+    R.run[lane] = v;
+    __syncwarp();
+    return __shfl_sync(kAll, incl, 31);
+}
+
+// Images of a row that the cells cx - S_x ... cx + S_x touch.
+__device__ __forceinline__ int nbr_images(const CellGrid& g, int cx)
+{
+    if (!g.pbc[0]) return 1;
+    const int ncx = g.nc[0];
+    int lo = 0, hi = 0;
+    for (int x = cx - g.S[0]; x < 0; x += ncx) --lo;
+    for (int x = cx + g.S[0]; x >= ncx; x -= ncx) ++hi;
+    return hi - lo + 1;
+}
+
+// The distance test: j at the cell offset (dx, dy, dz) from i's cell.  Explicit roundings:
+// every kernel decides alike.
+template <typename real>
+__device__ __forceinline__ real nbr_r2(const PosRec<real>& ri, const PosRec<real>& rj, int dx, int dy, int dz, real lx,
+                                       real ly, real lz)
+{
+    const real x = rj.x - fma(-(real)dx, lx, ri.x), y = rj.y - fma(-(real)dy, ly, ri.y),
+               z = rj.z - fma(-(real)dz, lz, ri.z);
+    return fma(z, z, fma(y, y, x * x));
+}
+
+__device__ __forceinline__ uint32_t nbr_entry(int k, int dx, int dy, int dz)
+{
+    return (uint32_t)k | ((uint32_t)((dx + 2) | ((dy + 2) << 3) | ((dz + 2) << 6)) << kJBits);
+}
+
+// particle i's counts, and its fixed-point lines at zero for the evaluation
+template <typename real>
+__device__ __forceinline__ void nbr_finish(const NeighborArgs<real>& a, int i, int nr, int na)
+{
+    a.cntR[i] = nr;
+    a.cntA[i] = na;
+    if (a.accF) {
+        ulonglong2* zl = reinterpret_cast<ulonglong2*>(a.accF + (size_t)i * 4);
+        zl[0] = zl[1] = make_ulonglong2(0ull, 0ull);
     }
-    if (a.accW && lane < 6) {
-        reinterpret_cast<ulonglong2*>(a.accW + (size_t)i * 12)[lane] = make_ulonglong2(0ull, 0ull);
+    if (a.accW) {
+        ulonglong2* zl = reinterpret_cast<ulonglong2*>(a.accW + (size_t)i * 12);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) zl[k] = make_ulonglong2(0ull, 0ull);
     }
 }
 
-// Work items up to which the warp-per-particle kernel runs.  Measured on water boxes
-// (neighbour stage, ms): 16 items 0.027 (warp) against 0.084 (thread per particle),
-// 40 items 0.033 / 0.071, 79 items 0.055 / 0.066, 118 items 0.076 / 0.070, 157 items
-// 0.097 / 0.073.
-constexpr int kNbrWarpMaxItems = 96;
+// One warp for P consecutive sorted particles, one after the other; those of one cell share
+// the run table and the loads of the candidates.  The lanes test 32 of a particle's
+// candidates at a time, and ballots compact the accepted ones in candidate order.  With
+// few particles the time is that of one warp's chain of steps, so P is 1; with more, P
+// spreads the chain's loads over several particles.  A block takes kBlock / 32 * P particles
+// of one work item.
+template <typename real, int P>
+__global__ void __launch_bounds__(kBlock) k_neighbors_warp(NeighborArgs<real> a)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kPerItem = 32 / P;  // blocks per work item
+    __shared__ NbrRuns run_tables[kBlock / 32];
+    __shared__ PosRec<real> recs[kBlock / 32][P];
+    const int item = (int)blockIdx.x / kPerItem;
+    if (item >= a.counts->n_items) return;
+    const WorkItem it = a.items[item];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = it.begin + (((int)blockIdx.x % kPerItem) * (kBlock / 32) + warp) * P;
+    const int many = min(P, it.end - first);
+    if (many <= 0) return;  // warp-uniform
+    NbrRuns& R = run_tables[warp];
+    const ReqInfo& q = a.reqs[it.req];
+    const ModelDesc<real>& md = a.models[q.model];
+    const CellGrid& g = q.g;
+    const int T = md.T;
+    const real* __restrict__ tabR = md.params + md.off.rcR2;
+    const real* __restrict__ tabA = md.params + md.off.rcA2;
+    const real cR1 = tabR[0], cA1 = tabA[0];  // the one pair type of a one-type model
+    const real lx = (real)g.len[0], ly = (real)g.len[1], lz = (real)g.len[2];
+    const unsigned below = (1u << lane) - 1u;
+    const uint32_t stride = (uint32_t)a.n;
+    int cell = -1, my_nr = 0, my_na = 0;  // of particle first + lane
+    if (lane < many) {
+        recs[warp][lane] = a.rec[first + lane];
+        cell = min(max(a.cell_s[first + lane] - q.cell_base, 0), g.ncell - 1);  // clamped as in k_neighbors
+    }
+    __syncwarp();
+    for (int p0 = 0, p1; p0 < many; p0 = p1) {
+        const int c = __shfl_sync(kAll, cell, p0);
+        p1 = p0 + __popc(__ballot_sync(kAll, lane < many && lane >= p0 && cell == c));  // sorted: one stretch
+        const int cx = c % g.nc[0], row = c / g.nc[0], cy = row % g.nc[1], cz = row / g.nc[1];
+        const int images = nbr_images(g, cx), runs = images * (2 * g.S[1] + 1) * (2 * g.S[2] + 1);
+        for (int r0 = 0; r0 < runs; r0 += kNbrRuns) {
+            const int total = nbr_runs(R, g, q.cell_base, a.cell_start, cx, cy, cz, images, r0, runs);
+            NbrCursor cur;
+            NbrCand cn = {0, 0, 0, 0};
+            PosRec<real> rn = recs[warp][0];
+            if (lane < total) {
+                cn = cur.at(R, lane, a.cell_s, cx);
+                rn = ldg_rec(a.rec + cn.k);
+            }
+            for (int f0 = 0; f0 < total; f0 += 32) {
+                const NbrCand cc = cn;
+                const PosRec<real> rj = rn;
+                if (f0 + 32 + lane < total) {  // the next 32, in flight during the tests
+                    cn = cur.at(R, f0 + 32 + lane, a.cell_s, cx);
+                    rn = ldg_rec(a.rec + cn.k);
+                }
+                // (an inconsistent cell list, which k_cell_rank reports, may hold a foreign cell here)
+                const bool own = f0 + lane < total && (unsigned)(cc.dx + g.S[0]) <= (unsigned)(2 * g.S[0]);
+                const int self = cc.dx == 0 && cc.dy == 0 && cc.dz == 0 ? cc.k : -1;
+                const real ox = (real)cc.dx, oy = (real)cc.dy, oz = (real)cc.dz;
+                const uint32_t ent = nbr_entry(cc.k, cc.dx, cc.dy, cc.dz);
+#pragma unroll 2
+                for (int p = p0; p < p1; ++p) {
+                    const PosRec<real> ri = recs[warp][p];
+                    const int i = first + p;
+                    const real x = rj.x - fma(-ox, lx, ri.x), y = rj.y - fma(-oy, ly, ri.y), z = rj.z - fma(-oz, lz, ri.z);
+                    const real r2 = fma(z, z, fma(y, y, x * x));
+                    real cR = cR1, cA = cA1;
+                    if (T > 1) {
+                        cR = tabR[ri.t * T + rj.t];
+                        cA = tabA[ri.t * T + rj.t];
+                    }
+                    const bool ok = own & (self != i);
+                    const bool inR = ok & (r2 < cR), inA = ok & (r2 < cA);
+                    const unsigned mR = __ballot_sync(kAll, inR), mA = __ballot_sync(kAll, inA);
+                    const int nr = P == 1 ? my_nr : __shfl_sync(kAll, my_nr, p);
+                    const int na = P == 1 ? my_na : __shfl_sync(kAll, my_na, p);
+                    const int sR = nr + __popc(mR & below), sA = na + __popc(mA & below);
+                    if (inR && sR < a.mnR) a.nlR[(uint32_t)sR * stride + (uint32_t)i] = ent;
+                    if (inA && sA < a.mnA) a.nlA[(uint32_t)sA * stride + (uint32_t)i] = ent;
+                    if (P == 1 || lane == p) {
+                        my_nr += __popc(mR);
+                        my_na += __popc(mA);
+                    }
+                }
+            }
+        }
+    }
+    if (lane < many) nbr_finish(a, first + lane, my_nr, my_na);
+    const int mxR = __reduce_max_sync(kAll, my_nr), mxA = __reduce_max_sync(kAll, my_na);
+    if (lane == 0) {
+        atomicMax(&a.maxcnt[0], mxR);
+        atomicMax(&a.maxcnt[1], mxA);
+    }
+}
+
+// Which kernel.  Measured (FP32; one warp per particle / per eight particles / one thread per
+// particle): water at 4 items 14 / 30 / 48 us, at 24 items 19 / 39 / 67, at 782 items
+// 254 / 130 / 103; a 60,000-particle nanowire (469 items, a dense core) 122 / 69 / 104; a
+// 50,000-particle monolayer (392 items, 1.2 particles to a cell, so that nothing is
+// shared between a warp's particles) 73 / 36 / 25.  FP64 tests every pair in FP64 in the warp
+// kernels and screens in FP32 in the other (782 items: 1217 / 1034 / 223 us).
+int neighbor_form(int items_cap, int n, int ncell, bool fp64)
+{
+    if (items_cap <= 90) return 1;
+    return !fp64 && items_cap <= 512 && n >= 2 * ncell ? 8 : 0;
+}
 
 // FP64 form: the FP32 copies of the sorted records that screen the distance tests
 // of k_neighbors (one conversion per particle instead of per candidate)
@@ -653,13 +794,13 @@ __global__ void __launch_bounds__(kBlock) k_round_records(const PlanCounts* __re
 }
 
 template <typename real>
-cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, size_t smem, cudaStream_t st)
+cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, int form, size_t smem, cudaStream_t st)
 {
     // the kernels index the slot-major lists with 32-bit slot * n + i
     if ((unsigned long long)(a.mnR > a.mnA ? a.mnR : a.mnA) * (unsigned long long)a.n > (1ull << 32))
         return cudaErrorInvalidValue;
-    if (items_cap <= kNbrWarpMaxItems)  // FP64 here tests every pair in FP64
-        return launch_k(k_neighbors_warp<real>, items_cap * (kBlock / kNbrWarpParticles), kBlock, smem, st, a);
+    if (form == 1) return launch_k(k_neighbors_warp<real, 1>, items_cap * 32, kBlock, 0, st, a);
+    if (form == 8) return launch_k(k_neighbors_warp<real, 8>, items_cap * 4, kBlock, 0, st, a);
     if constexpr (sizeof(real) == 8) {
         if (a.rec32) {
             const cudaError_t e = launch_k(k_round_records, (a.n + kBlock - 1) / kBlock, kBlock, 0, st, a.counts, a.rec,
@@ -679,7 +820,7 @@ cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, size_t 
                                                  const ReqInfo*, const ModelDesc<real>*, const double*,           \
                                                  const int*, int*, PosRec<real>*, int*, int*, int*, int*, int*,   \
                                                  int*, int*, int*, PosRec<real>*, int*, cudaStream_t);            \
-    template cudaError_t launch_neighbors<real>(const NeighborArgs<real>&, int, size_t, cudaStream_t);
+    template cudaError_t launch_neighbors<real>(const NeighborArgs<real>&, int, int, size_t, cudaStream_t);
 NEP_INSTANTIATE(float)
 NEP_INSTANTIATE(double)
 #undef NEP_INSTANTIATE

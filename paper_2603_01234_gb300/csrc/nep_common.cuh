@@ -296,8 +296,12 @@ cudaError_t launch_kick_drift_bin(const PlanCounts* counts, int items_cap, const
                                   double* vel, const double* force, int* cell_of, PosRec<real>* rec_user,
                                   int* cell_count, int* err, cudaStream_t st);
 
+// The neighbour kernel of a batch of n particles in ncell cells: the particles that a warp
+// takes (1 or 8), or 0 for one thread per particle.
+int neighbor_form(int items_cap, int n, int ncell, bool fp64);
+
 template <typename real>
-cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, size_t smem, cudaStream_t st);
+cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, int form, size_t smem, cudaStream_t st);
 
 // Shape-dispatched evaluation; returns cudaErrorInvalidValue for an uncompiled shape.
 // mb_desc / mb_force / ch_force: the variants of the thread-per-particle kernels
