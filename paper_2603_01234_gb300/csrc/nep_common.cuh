@@ -225,6 +225,22 @@ constexpr int kGroup = 32;
 // touching memory out of bounds.
 constexpr int kErrCellList = 4;
 
+// Where the totals of request r go: all ten together, and the caller's own arrays (either may
+// be absent).
+struct TotalsOut {
+    double* all = nullptr;     // [requests][10]: E, W[9]
+    double* energy = nullptr;  // [requests]
+    double* virial = nullptr;  // [requests][9]
+#ifdef __CUDACC__
+    __device__ __forceinline__ void write(int r, int t, double v) const
+    {
+        all[(size_t)r * 10 + t] = v;
+        if (energy && t == 0) energy[r] = v;
+        if (virial && t > 0) virial[(size_t)r * 9 + t - 1] = v;
+    }
+#endif
+};
+
 template <typename real>
 struct EvalArgs {
     int n, mnR, mnA;            // n: the list / array stride (particle capacity)
@@ -258,7 +274,7 @@ struct EvalArgs {
     unsigned int* gcounter;     // [items] last-block counters of the item groups, at each
                                 // group's first item (self-resetting)
     unsigned int* icounter;     // [items] group kernels: finished blocks of each item (self-resetting)
-    double* totals;             // [requests][10]: E, W[9]
+    TotalsOut totals;           // per request: E, W[9]
     int* err = nullptr;         // the error word (kErrCellList on an inconsistent cell list)
     // MD: the step's closing half-kick applied by the output pass as soon as F_i is
     // final, v_i <- half_kick(v_i, kick_half_dt, F_i, kick_im[t_i]), with the same
