@@ -470,16 +470,15 @@ int ensure_cells(nep_model* m, int ncell)
     // the scan leaves the counters of the cells it covers zero for the next build.  A
     // new buffer starts with anything in it and a failed build may leave counts behind,
     // so both are cleared over their whole capacity: a buffer grows by a quarter at
-    // least, and a later grid may reach cells that this one does not
-    const void* c0 = m->cell_count.p;
-    const void* f0 = m->cell_fill.p;
-    const void* b0 = m->block_off.p;
+    // least, and a later grid may reach cells that this one does not.  A new buffer is
+    // told by its capacity: its address may well be the freed one's
+    const size_t c0 = m->cell_count.cap, f0 = m->cell_fill.cap, b0 = m->block_off.cap;
     NEP_TRY(m->cell_count.ensure(sizeof(int) * ncell));
     NEP_TRY(m->cell_local.ensure(sizeof(int) * ncell));
     NEP_TRY(m->block_off.ensure(sizeof(int) * (kScanItems + 1)));
     NEP_TRY(m->cell_fill.ensure(sizeof(int) * ncell));
     NEP_TRY(m->cell_start.ensure(sizeof(int) * (ncell + 1)));
-    if (m->cells_dirty || m->cell_count.p != c0 || m->cell_fill.p != f0 || m->block_off.p != b0) {
+    if (m->cells_dirty || m->cell_count.cap != c0 || m->cell_fill.cap != f0 || m->block_off.cap != b0) {
         m->cells_dirty = true;
         NEP_CUDA(cudaMemsetAsync(m->cell_count.p, 0, m->cell_count.cap, m->cur));
         NEP_CUDA(cudaMemsetAsync(m->cell_fill.p, 0, m->cell_fill.cap, m->cur));

@@ -33,3 +33,22 @@ def test_grids_within_a_grown_buffer(nep_lib, precision):
         np.testing.assert_array_equal(got["force"], want["force"])
         np.testing.assert_array_equal(got["virial"], want["virial"])
     m.close()
+
+
+def test_fresh_handles_on_used_memory(nep_lib):
+    """Handles created on memory that earlier ones filled and gave back, each taken through
+    small grids of growing size: a buffer that is freed and allocated anew often comes back
+    at the same address, with other contents behind its old end."""
+    model = water_model()
+    rng = np.random.default_rng(5)
+    sizes = [64, 90, 130, 200, 300, 420, 150, 640, 800, 1000]
+    systems = [inputs.water_box(n, seed=300 + n) for n in sizes]
+    want = {}
+    for rep in range(12):
+        m = binding.Model(model, "fp32")
+        for k in rng.permutation(len(systems)):
+            got = m.compute(systems[k])
+            ref = want.setdefault(int(k), got)
+            assert got["energy"] == ref["energy"]
+            np.testing.assert_array_equal(got["force"], ref["force"])
+        m.close()
