@@ -46,7 +46,7 @@ struct GroupTile {
     static constexpr int ROW = (GS + 24) / 4 % 2 ? GS + 24 : GS + 28;
     static constexpr int PSI = 28;
     static constexpr int TILE = kG * ROW;
-    static constexpr int USED = TILE + NA * PSI;
+    static constexpr int USED = TILE + NA * PSI + 16;  // and PairFrame's table
     static constexpr int SIZE = (USED + 23) / 32 * 32 + 8;
     static_assert(SIZE >= USED, "group size");
 };
@@ -74,6 +74,48 @@ __device__ __forceinline__ real group_sum(real v)
     return v;
 }
 
+// Pair vectors of one particle.  FP64: r_i moved by the five possible cell offsets per axis,
+// looked up in shared memory, so that a component is one subtraction (the conversion of the
+// offset and the multiply-add would each cost as much on the FP64 pipe).
+template <typename real>
+struct PairFrame;
+template <>
+struct PairFrame<float> {
+    float len[3];
+    PosRec<float> ri;
+    __device__ __forceinline__ PairFrame(const CellGrid& g, const PosRec<float>& r, float*, int) : ri(r)
+    {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) len[k] = (float)g.len[k];
+    }
+    __device__ __forceinline__ void vec(const PosRec<float>& rj, uint32_t e, float& dx, float& dy, float& dz) const
+    {
+        pair_vec(len, ri, rj, e, dx, dy, dz);
+    }
+};
+template <>
+struct PairFrame<double> {
+    const double* moved;  // [3][5]
+    __device__ __forceinline__ PairFrame(const CellGrid& g, const PosRec<double>& r, double* table, int lane)
+        : moved(table)
+    {
+        if (lane < 5) {
+            const double d = (double)(2 - lane);
+            table[lane] = fma(d, g.len[0], r.x);
+            table[5 + lane] = fma(d, g.len[1], r.y);
+            table[10 + lane] = fma(d, g.len[2], r.z);
+        }
+        __syncwarp();
+    }
+    __device__ __forceinline__ void vec(const PosRec<double>& rj, uint32_t e, double& dx, double& dy, double& dz) const
+    {
+        const uint32_t code = e >> kJBits;
+        dx = rj.x - moved[code & 7u];
+        dy = rj.y - moved[5 + ((code >> 3) & 7u)];
+        dz = rj.z - moved[10 + ((code >> 6) & 7u)];
+    }
+};
+
 // A pair's geometry from the list entry.
 template <typename real>
 struct Pair {
@@ -81,13 +123,12 @@ struct Pair {
     int j, tj;
 };
 template <typename real>
-__device__ __forceinline__ Pair<real> make_pair(const PosRec<real>& ri, const PosRec<real>& rj, uint32_t e,
-                                                const real (&len)[3])
+__device__ __forceinline__ Pair<real> make_pair(const PairFrame<real>& frame, const PosRec<real>& rj, uint32_t e)
 {
     Pair<real> p;
     p.j = (int)(e & kJMask);
     p.tj = rj.t;
-    pair_vec(len, ri, rj, e, p.dx, p.dy, p.dz);
+    frame.vec(rj, e, p.dx, p.dy, p.dz);
     const real r2 = norm2(p.dx, p.dy, p.dz);
     p.inv_r = rsqrt_r(r2);
     p.r = r2 * p.inv_r;
@@ -119,8 +160,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
     // groups past the item's end follow its last particle with empty lists and write nothing
     const bool live = first + grp < it.end;
     const int i = live ? first + grp : it.end - 1;
-    const real len[3] = {(real)rq.g.len[0], (real)rq.g.len[1], (real)rq.g.len[2]};
     const PosRec<real> ri = a.rec[i];
+    const PairFrame<real> frame(rq.g, ri, psi + NA * GT::PSI, gl);
     const int ti = ri.t;
     const int cR = live ? min(a.cntR[i], a.mnR) : 0, cA = live ? min(a.cntA[i], a.mnA) : 0;
     const size_t n = (size_t)a.n;
@@ -133,7 +174,8 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
     static_assert(GT::TILE >= 144 && ND + 2 <= 40, "network scratch");
 
     // ---- radial descriptors (Eq. 3, 6-8) ----
-    real qr[NR];
+    real q_own = real(0);  // q_n of lane n < NR
+    static_assert(NR <= kG, "a lane per radial descriptor");
     {
         const uint32_t* nl = a.nlR + (size_t)gl * n + i;
         const int cl = (cR - gl + kG - 1) / kG;  // this lane's slots (none: <= 0)
@@ -143,32 +185,32 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
             for (int k = 0; k < KR; ++k) f[k] = real(0);
             const real inv_rc = P[off.rcRi], inv_lo = P[off.rcRl];
             walk4(nl, kG * n, cl, [&](uint32_t e) {
-                const Pair<real> p = make_pair(ri, a.rec[e & kJMask], e, len);
+                const Pair<real> p = make_pair(frame, a.rec[e & kJMask], e);
                 basis_acc<real, KR>(p.r, inv_rc, inv_lo, f, hs);
             });
             hs = group_sum(hs);
 #pragma unroll
             for (int k = 0; k < KR; ++k) f[k] = group_sum(f[k]) + hs;
-            const real* c = P + off.cR;
+            // lane n has row n
+            const int nn = min(gl, NR - 1);
+            const real* c = P + off.cR + nn * KR;
+            real g = real(0);
 #pragma unroll
-            for (int nn = 0; nn < NR; ++nn) {
-                real g = real(0);
+            for (int k = 0; k < KR; ++k) g = fma(c[k], f[k], g);
+            if constexpr (kF32) {
+                const real* cl_ = P + off.cRl + nn * KR;
+                real gl_ = real(0);
 #pragma unroll
-                for (int k = 0; k < KR; ++k) g = fma(c[nn * KR + k], f[k], g);
-                if constexpr (kF32) {
-                    const real* cl_ = P + off.cRl;
-                    real gl_ = real(0);
-#pragma unroll
-                    for (int k = 0; k < KR; ++k) gl_ = fma(cl_[nn * KR + k], f[k], gl_);
-                    g += gl_;
-                }
-                qr[nn] = g;
+                for (int k = 0; k < KR; ++k) gl_ = fma(cl_[k], f[k], gl_);
+                g += gl_;
             }
+            q_own = g;
         } else {
+            real qr[NR];
 #pragma unroll
             for (int nn = 0; nn < NR; ++nn) qr[nn] = real(0);
             walk4(nl, kG * n, cl, [&](uint32_t e) {
-                const Pair<real> p = make_pair(ri, a.rec[e & kJMask], e, len);
+                const Pair<real> p = make_pair(frame, a.rec[e & kJMask], e);
                 const int tp = ti * T + p.tj;
                 real f[KR];
                 basis<real, KR>(p.r, P[off.rcRi + tp], P[off.rcRl + tp], f);
@@ -182,7 +224,10 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
                 }
             });
 #pragma unroll
-            for (int nn = 0; nn < NR; ++nn) qr[nn] = group_sum(qr[nn]);
+            for (int nn = 0; nn < NR; ++nn) {
+                qr[nn] = group_sum(qr[nn]);
+                if (gl == nn) q_own = qr[nn];
+            }
         }
     }
 
@@ -209,7 +254,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
 #pragma unroll
             for (int k = 0; k < GT::GS; ++k) g[k] = real(0);
             if (ok) {
-                const Pair<real> p = make_pair(ri, rc, ec, len);
+                const Pair<real> p = make_pair(frame, rc, ec);
                 const int tp = ti * T + p.tj;
                 real hf, t[KA];
                 cheb_T<real, KA>(p.r, P[off.rcAi + tp], P[off.rcAl + tp], hf, t);
@@ -270,10 +315,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
             sq[NR + 5 * NA + gl] = ql[0] * ql[0];
         }
     }
-    if (gl == 0) {
-#pragma unroll
-        for (int nn = 0; nn < NR; ++nn) sq[nn] = qr[nn];
-    }
+    if (gl < NR) sq[gl] = q_own;
     __syncwarp();
 
     // ---- network (Eq. 2) and dU/dq ----
@@ -417,7 +459,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(real) == 4 ? 4 : 3) k_descripto
 #pragma unroll
         for (int k = 0; k < 12; ++k) out[k] = real(0);
         if (s < cA) {
-            const Pair<real> p = make_pair(ri, rc, ec, len);
+            const Pair<real> p = make_pair(frame, rc, ec);
             const int tij = ti * T + p.tj;
             real hf, hdf, hdx, t[KA], dt[KA];
             cheb_dT<real, KA>(p.r, P[off.rcAi + tij], P[off.rcAl + tij], hf, hdf, hdx, t, dt);
@@ -497,7 +539,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
 {
     constexpr int KRP = (KR + 3) & ~3;
     constexpr bool kF32 = sizeof(real) == 4;
-    constexpr int ROW = 12, GROUP = kG * ROW + 8;  // 104 = 8 mod 32 (see GroupTile)
+    constexpr int ROW = 12, GROUP = kG * ROW + (kF32 ? 8 : 40);  // 8 mod 32 (see GroupTile); FP64: PairFrame's table
     __shared__ __align__(16) real smem[kGP * GROUP];
     __shared__ bool last;
     const int item = (int)blockIdx.x / kG;
@@ -515,8 +557,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
     const bool live = first + grp < it.end;
     const int i = live ? first + grp : it.end - 1;
     const size_t n = (size_t)a.n;
-    const real len[3] = {(real)rq.g.len[0], (real)rq.g.len[1], (real)rq.g.len[2]};
     const PosRec<real> ri = a.rec[i];
+    const PairFrame<real> frame(rq.g, ri, tile + kG * ROW, gl);
     const int ti = ri.t;
     const int cR = live ? min(a.cntR[i], a.mnR) : 0;
     const int most = __reduce_max_sync(kFull, cR);
@@ -545,7 +587,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
             const int j = (int)(ec & kJMask);
             real eji[KRP], eij[KRP];
             loadN<real, KRP>(a.e + (size_t)j * a.e_stride + ti * KRP, eji);
-            const Pair<real> p = make_pair(ri, a.rec[j], ec, len);
+            const Pair<real> p = make_pair(frame, a.rec[j], ec);
             if (T == 1) {
 #pragma unroll
                 for (int k = 0; k < KRP; ++k) eij[k] = ei1[k];
@@ -615,7 +657,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
             const uint32_t back = (uint32_t)i | ((0x124u - (ea >> kJBits)) << kJBits);
             const int cj = min(a.cntA[j], a.mnA);
             real dx, dy, dz;
-            pair_vec(len, ri, a.rec[j], ea, dx, dy, dz);
+            frame.vec(a.rec[j], ea, dx, dy, dz);
             const real* fi = a.fang + ((size_t)s * n + i) * 3;
             real fj[3] = {real(0), real(0), real(0)};
             for (int t = 0; t < cj; ++t)

@@ -6,6 +6,7 @@
 
 #include "nep_common.cuh"
 #include "poly32.cuh"
+#include "poly64.cuh"
 #include "sh_poly.cuh"
 
 namespace nep {
@@ -18,7 +19,8 @@ constexpr int kNLM = 24;
 // The cutoff of Eq. 8 halved, f_c / 2, and its derivative halved, f_c' / 2, at
 // x = r / r_c in [0, 1].  FP32 evaluates the polynomials of poly32.cuh
 // (the hardware sine and cosine err by about 1e-7 with a consistent sign, which
-// summed over pairs biases the energy); FP64 uses the accurate sincospi.
+// summed over pairs biases the energy), FP64 those of poly64.cuh (on this range they take
+// half the FP64 instructions of cospi and sincospi, and the FP64 kernels are bound by those).
 __device__ __forceinline__ float cut_half(float x)
 {
     const float y = x - 0.5f;
@@ -26,7 +28,8 @@ __device__ __forceinline__ float cut_half(float x)
 }
 __device__ __forceinline__ double cut_half(double x)
 {
-    return 0.25 + 0.25 * cospi(x);
+    const double y = x - 0.5;
+    return fma(-y, cut_p64(y * y), 0.25);
 }
 __device__ __forceinline__ void cut_half_d(float x, float inv_rc, float* hf, float* hdf)
 {
@@ -37,10 +40,10 @@ __device__ __forceinline__ void cut_half_d(float x, float inv_rc, float* hf, flo
 }
 __device__ __forceinline__ void cut_half_d(double x, double inv_rc, double* hf, double* hdf)
 {
-    double s, c;
-    sincospi(x, &s, &c);
-    *hf = 0.25 + 0.25 * c;
-    *hdf = (-0.25 * 3.14159265358979323846) * inv_rc * s;
+    const double y = x - 0.5;
+    const double z = y * y;
+    *hf = fma(-y, cut_p64(z), 0.25);
+    *hdf = -cut_q64(z) * inv_rc;
 }
 
 // Chebyshev basis f_k(r) of Eq. 7 with the cutoff of Eq. 8, k = 0..K-1, by the
@@ -382,7 +385,28 @@ __device__ __forceinline__ float rsqrt_r(float x)
     const float e = fmaf(-x, y * y, 1.0f);
     return fmaf(0.5f * y, e, y);
 }
-__device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
+// Conversions between FP64 and FP32 by moving bits, for values of FP32's normal range (the
+// conversion instructions run at the FP64 rate): FP64 truncated to FP32, and FP32 widened.
+__device__ __forceinline__ bool fp32_range(int hi) { return (unsigned)(hi - 0x38100000) < 0x0fe00000u; }
+__device__ __forceinline__ float narrow_bits(double x)
+{
+    return __int_as_float((int)(((unsigned)__double2hiint(x) - 0x38000000u) << 3 | (unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double widen_bits(float x)
+{
+    const unsigned b = (unsigned)__float_as_int(x);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// FP64: the FP32 estimate refined by one step of Householder's third-order iteration,
+// y' = y + y e (1/2 + 3/8 e), e = 1 - x y^2 (|e| < 1e-6, so its error is below e^3).
+__device__ __forceinline__ double rsqrt_r(double x)
+{
+    if (!fp32_range(__double2hiint(x))) return rsqrt(x);
+    const double y = widen_bits(rsqrtf(narrow_bits(x)));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
 // tanh in FP32.  Each hidden unit's pre-activation keeps one sign over most
 // particles, so an activation whose rounding error leans one way on part of its
@@ -404,7 +428,34 @@ __device__ __forceinline__ float tanh_r(float x)
     r = fmaf(r, fmaf(-d, r, 1.0f), r);
     return copysignf((1.0f - e) * r, x);
 }
-__device__ __forceinline__ double tanh_r(double x) { return tanh(x); }
+// FP64: tanh a = -m / (2 + m), m = exp(-2a) - 1, a = |x|.  exp(-2a) = 2^(n/32) exp(r) with
+// |r| <= ln 2 / 64: 2^(n/32) from a table, exp(r) - 1 by its series to r^6 (the next term is
+// below 4e-18); the reciprocal of 2 + m in (1, 2] is an FP32 one refined to third order.  No
+// cancellation: for small a, n = 0 and m is the series alone.
+__device__ __forceinline__ double tanh_r(double x)
+{
+    const int top = __double2hiint(x) & 0x7fffffff;
+    if (top >= 0x40340000) return top >= 0x7ff00000 ? tanh(x) : copysign(1.0, x);  // |x| >= 20
+    const double t = -2.0 * fabs(x);
+    constexpr double kRound = 6755399441055744.0;  // 3 2^51: adding it rounds to an integer
+    const double s = fma(t, kLn2Inv, kRound);
+    const int n = __double2loint(s);
+    const double nd = s - kRound;
+    const double r = fma(-nd, kLn2Lo, fma(-nd, kLn2Hi, t));
+    double p = fma(r, 1.0 / 720.0, 1.0 / 120.0);
+    p = fma(p, r, 1.0 / 24.0);
+    p = fma(p, r, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(p * r, r, r);  // exp(r) - 1
+    const double b = __ldg(kExp2Table + (n & 31));
+    const double em = __hiloint2double(__double2hiint(b) + ((n >> 5) << 20), __double2loint(b));
+    const double m = fma(em, p + __ldg(kExp2Rest + (n & 31)), em - 1.0);
+    const double d = 2.0 + m;
+    const double y = widen_bits(__fdividef(1.0f, narrow_bits(d)));
+    const double e = fma(-d, y, 1.0);
+    const double h = -m * fma(y, fma(e, e, e), y);
+    return __hiloint2double(__double2hiint(h) | (__double2hiint(x) & (int)0x80000000), __double2loint(h));
+}
 
 // a product that is never contracted into a multiply-add
 __device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
