@@ -353,7 +353,7 @@ __device__ __forceinline__ void force_radial(const EvalArgs<real>& a, const real
         const int j = (int)(e & kJMask);
         const PosRec<real> rj = a.rec[j];
         real eji[KRP];
-        loadN<real, KRP>(a.e + (size_t)j * a.e_stride + ti * KRP, eji);
+        load_grad<real, KRP>(a.e + (size_t)j * a.e_stride + ti * KRP, eji);
         real dx, dy, dz;
         pair_vec(c.len, c.ri, rj, e, dx, dy, dz);
         const real r2 = norm2(dx, dy, dz);
@@ -385,12 +385,12 @@ __device__ __forceinline__ void force_radial(const EvalArgs<real>& a, const real
     const size_t stride = (size_t)a.n;
     if (T == 1) {
         real ei1[KRP];  // the one partner type's vector
-        loadN<real, KRP>(e_i, ei1);
+        load_grad<real, KRP>(e_i, ei1);
         walk_chunk<CH>(nl, stride, cnt, [&](uint32_t e) { radial_pair(e, ei1); });
     } else {
         walk_chunk<CH>(nl, stride, cnt, [&](uint32_t e) {
             real eij[KRP];
-            loadN<real, KRP>(e_i + a.rec[e & kJMask].t * KRP, eij);
+            load_grad<real, KRP>(e_i + a.rec[e & kJMask].t * KRP, eij);
             radial_pair(e, eij);
         });
     }

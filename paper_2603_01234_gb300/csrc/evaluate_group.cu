@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
     const real* e_i = a.e + (size_t)i * a.e_stride;
     const uint32_t* nl = a.nlR + i;
     real ei1[KRP];
-    if (T == 1) loadN<real, KRP>(e_i, ei1);
+    if (T == 1) load_grad<real, KRP>(e_i, ei1);
     // FP32: component c < 9 of (F, symmetric W) is the sum over the pairs, in slot order, of
     // the product of row entries ia and ib; lane c has component c, lane 0 also component 8.
     // FP64: each lane sums its pairs' components.
@@ -574,25 +574,35 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
     real F[3] = {real(0), real(0), real(0)}, W[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) W[k] = real(0);
+    // the list two rounds ahead, the neighbour's record and gradient vector one round ahead
     uint32_t e = gl < cR ? nl[(size_t)gl * n] : 0u;
     uint32_t e2 = kG + gl < cR ? nl[(size_t)(kG + gl) * n] : 0u;
+    PosRec<real> rj = a.rec[e & kJMask];
+    real ej[KRP];
+    load_grad<real, KRP>(a.e + (size_t)(e & kJMask) * a.e_stride + ti * KRP, ej);
     for (int s0 = 0; s0 < most; s0 += kG) {
         const int s = s0 + gl;
         const uint32_t ec = e;
+        const PosRec<real> rc = rj;
+        real eji[KRP];
+#pragma unroll
+        for (int k = 0; k < KRP; ++k) eji[k] = ej[k];
         e = e2;
         e2 = s + 2 * kG < cR ? nl[(size_t)(s + 2 * kG) * n] : 0u;
+        if (s0 + kG < most) {
+            rj = a.rec[e & kJMask];
+            load_grad<real, KRP>(a.e + (size_t)(e & kJMask) * a.e_stride + ti * KRP, ej);
+        }
         real fs = real(0), ux = real(0), uy = real(0), uz = real(0), wx = real(0), wy = real(0), wz = real(0);
         real dx = real(0), dy = real(0), dz = real(0);
         if (s < cR) {
-            const int j = (int)(ec & kJMask);
-            real eji[KRP], eij[KRP];
-            loadN<real, KRP>(a.e + (size_t)j * a.e_stride + ti * KRP, eji);
-            const Pair<real> p = make_pair(frame, a.rec[j], ec);
+            real eij[KRP];
+            const Pair<real> p = make_pair(frame, rc, ec);
             if (T == 1) {
 #pragma unroll
                 for (int k = 0; k < KRP; ++k) eij[k] = ei1[k];
             } else {
-                loadN<real, KRP>(e_i + p.tj * KRP, eij);
+                load_grad<real, KRP>(e_i + p.tj * KRP, eij);
             }
             real f[KR], df[KR];
             const int tp = ti * T + p.tj;

@@ -360,6 +360,20 @@ __device__ __forceinline__ void loadN(const real* p, real* o)
     for (int k = N & ~3; k < N; ++k) o[k] = p[k];
 }
 
+// A gradient vector (N reals, rows 32-byte aligned when N = 8 floats) from global memory: eight
+// floats in one 256-bit load, whose one line look-up is what a gather costs.
+template <typename real, int N>
+__device__ __forceinline__ void load_grad(const real* p, real* o)
+{
+    if constexpr (sizeof(real) == 4 && N == 8) {
+        asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]), "=f"(o[4]), "=f"(o[5]), "=f"(o[6]), "=f"(o[7])
+                     : "l"(p));
+    } else {
+        loadN<real, N>(p, o);
+    }
+}
+
 // 1/sqrt(x): the hardware estimate refined by one Newton-Raphson step on
 // f(y) = y^-2 - x, y' = y + y (1 - x y^2) / 2.  The estimate's error has a small
 // consistent sign, which through |u| = |r| / r and the homogeneous harmonics would
