@@ -85,28 +85,34 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
     const int cR = min(a.cntR[i], a.mnR);
     if (T == 1) {
         // one pair type: q_n = sum_k c_nk (sum_j f_k(r_ij)), contracted once per bead;
-        // the pair sums are kept as eight partial sums (see walk8p)
-        real fp[8][KR], hp[8];
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-            hp[p] = real(0);
-#pragma unroll
-            for (int k = 0; k < KR; ++k) fp[p][k] = real(0);
-        }
+        // the pair sums are kept as eight partial sums, four at a time (see walk_half)
         const real inv_rc = P[off.rcRi], inv_lo = P[off.rcRl];
-        walk8p(a.nlR + i, (size_t)a.n, cR, [&](uint32_t e, int p) {
-            const PosRec<real> rj = a.rec[e & kJMask];
-            real dx, dy, dz;
-            pair_vec(len, ri, rj, e, dx, dy, dz);
-            const real r2 = norm2(dx, dy, dz);
-            const real r = r2 * rsqrt_r(r2);
-            basis_acc<real, KR>(r, inv_rc, inv_lo, fp[p], hp[p]);
-        });
-        const real hs = sum8(hp[0], hp[1], hp[2], hp[3], hp[4], hp[5], hp[6], hp[7]);
-        real fs[KR];
+        real fs[KR], hs = real(0);
 #pragma unroll
-        for (int k = 0; k < KR; ++k)
-            fs[k] = sum8(fp[0][k], fp[1][k], fp[2][k], fp[3][k], fp[4][k], fp[5][k], fp[6][k], fp[7][k]) + hs;
+        for (int k = 0; k < KR; ++k) fs[k] = real(0);
+#pragma unroll 1
+        for (int first = 0; first < 8; first += 4) {
+            real fp[4][KR], hp[4];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                hp[p] = real(0);
+#pragma unroll
+                for (int k = 0; k < KR; ++k) fp[p][k] = real(0);
+            }
+            walk_half(a.nlR + i, (size_t)a.n, cR, first, [&](uint32_t e, int p) {
+                const PosRec<real> rj = a.rec[e & kJMask];
+                real dx, dy, dz;
+                pair_vec(len, ri, rj, e, dx, dy, dz);
+                const real r2 = norm2(dx, dy, dz);
+                const real r = r2 * rsqrt_r(r2);
+                basis_acc<real, KR>(r, inv_rc, inv_lo, fp[p], hp[p]);
+            });
+            hs += (hp[0] + hp[1]) + (hp[2] + hp[3]);
+#pragma unroll
+            for (int k = 0; k < KR; ++k) fs[k] += (fp[0][k] + fp[1][k]) + (fp[2][k] + fp[3][k]);
+        }
+#pragma unroll
+        for (int k = 0; k < KR; ++k) fs[k] += hs;
         const real* c = P + off.cR;
 #pragma unroll
         for (int nn = 0; nn < NR; ++nn) {
@@ -123,32 +129,34 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
             q[nn] = g;
         }
     } else {
-        real qp[8][NR];  // eight partial sums (see walk8p)
+#pragma unroll 1
+        for (int first = 0; first < 8; first += 4) {  // eight partial sums, four at a time (see walk_half)
+            real qp[4][NR];
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
+            for (int p = 0; p < 4; ++p)
 #pragma unroll
-            for (int nn = 0; nn < NR; ++nn) qp[p][nn] = real(0);
-        walk8p(a.nlR + i, (size_t)a.n, cR, [&](uint32_t e, int p) {
-            const PosRec<real> rj = a.rec[e & kJMask];
-            real dx, dy, dz;
-            pair_vec(len, ri, rj, e, dx, dy, dz);
-            const real r2 = norm2(dx, dy, dz);
-            const real r = r2 * rsqrt_r(r2);
-            const int tp = ti * T + rj.t;
-            real f[KR];
-            basis<real, KR>(r, P[off.rcRi + tp], P[off.rcRl + tp], f);
-            const real* c = P + off.cR + tp * coef_stride(NR, KR);
+                for (int nn = 0; nn < NR; ++nn) qp[p][nn] = real(0);
+            walk_half(a.nlR + i, (size_t)a.n, cR, first, [&](uint32_t e, int p) {
+                const PosRec<real> rj = a.rec[e & kJMask];
+                real dx, dy, dz;
+                pair_vec(len, ri, rj, e, dx, dy, dz);
+                const real r2 = norm2(dx, dy, dz);
+                const real r = r2 * rsqrt_r(r2);
+                const int tp = ti * T + rj.t;
+                real f[KR];
+                basis<real, KR>(r, P[off.rcRi + tp], P[off.rcRl + tp], f);
+                const real* c = P + off.cR + tp * coef_stride(NR, KR);
 #pragma unroll
-            for (int nn = 0; nn < NR; ++nn) {
-                real g = real(0);
+                for (int nn = 0; nn < NR; ++nn) {
+                    real g = real(0);
 #pragma unroll
-                for (int k = 0; k < KR; ++k) g += c[nn * KR + k] * f[k];
-                qp[p][nn] += g;
-            }
-        });
+                    for (int k = 0; k < KR; ++k) g += c[nn * KR + k] * f[k];
+                    qp[p][nn] += g;
+                }
+            });
 #pragma unroll
-        for (int nn = 0; nn < NR; ++nn)
-            q[nn] = sum8(qp[0][nn], qp[1][nn], qp[2][nn], qp[3][nn], qp[4][nn], qp[5][nn], qp[6][nn], qp[7][nn]);
+            for (int nn = 0; nn < NR; ++nn) q[nn] += (qp[0][nn] + qp[1][nn]) + (qp[2][nn] + qp[3][nn]);
+        }
     }
 
     // ---- angular moments A_nlm (Eq. 5) ----
@@ -631,11 +639,11 @@ static cudaError_t launch_force_radial(const EvalArgs<float>& a, int nb, size_t 
 
 // FP32 batches up to this many work items run the group kernels (evaluate_group.cu).  Theirs
 // is the shorter latency, the thread-per-particle kernels' the fewer instructions: on
-// water the group kernels' two launches take 40 us at 4 items (82 us here), 51 at 24 (104)
+// water the group kernels' two launches take 37 us at 4 items (82 us here), 50 at 24 (104)
 // and then 0.53 us an item, and the ones here about 110 us until the chip is full at 456
 // items.  FP64 always runs the group kernels: bound by the FP64 pipe, they evaluate each
-// ordered angular pair once and do not spill (100,000-bead water 6.13 ms, with one thread
-// per particle and both directions of each pair evaluated 7.00 ms).
+// ordered angular pair once and do not spill (100,000-bead water 5.01 ms; one thread per
+// particle and both directions of each pair took 7.00 ms).
 constexpr int kGroupMaxItems = 200;
 
 bool evaluate_by_groups(int items_cap, bool fp64) { return fp64 || items_cap <= kGroupMaxItems; }

@@ -787,8 +787,9 @@ static cudaError_t launch_descriptor_group(const EvalArgs<real>& a, int nb, cuda
 template <typename real>
 cudaError_t group_set_smem()
 {
-    // FP64 rows of the second shape take more than the 48 KB a kernel gets unasked
+    // only the FP64 rows of the second shape take more than the 48 KB a kernel gets unasked
     auto set = [](auto* kernel, size_t bytes) {
+        if (bytes <= 48 * 1024) return cudaSuccess;
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
     cudaError_t e = cudaSuccess;

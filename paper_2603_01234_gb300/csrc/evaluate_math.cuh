@@ -297,46 +297,33 @@ __device__ __forceinline__ void walk_chunk(const uint32_t* nl, size_t stride, in
         if (s + u < cnt) body(q[u]);
 }
 
-// The walk in groups of eight with the entry's position in its group passed as the
-// second argument (0..7, a constant after unrolling), so that a body can keep eight
-// partial sums, one per slot number mod 8: each grows to an eighth of the total, which
-// cuts the FP32 rounding of a long accumulation at no extra instructions, and they are
-// the sums that the eight lanes of evaluate_group.cu form.
+// Half of a walk in groups of eight: the entries first ... first + 3 of every eight (first =
+// 0 or 4), with the position among the four as the body's second argument (0..3, a constant
+// after unrolling), so that a body can keep four partial sums.  The two halves' sums are
+// partial sums by slot number mod 8: each grows to an eighth of the total, which cuts the
+// FP32 rounding of a long accumulation, and they are the sums that the eight lanes of
+// evaluate_group.cu form.  (All eight at once cost the four-type monolayer, with six pairs a
+// particle, 1.5% of a step.)
 template <typename Body>
-__device__ __forceinline__ void walk8p(const uint32_t* nl, size_t stride, int cnt, Body&& body)
+__device__ __forceinline__ void walk_half(const uint32_t* nl, size_t stride, int cnt, int first, Body&& body)
 {
     auto ld = [&](int s) { return s < cnt ? nl[(size_t)s * stride] : 0u; };
-    uint32_t q[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) q[u] = ld(u);
-    int s = 0;
-    for (; s + 8 <= cnt; s += 8) {
-        uint32_t cur[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            cur[u] = q[u];
-            q[u] = ld(s + 8 + u);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) body(cur[u], u);
+    int s = first;
+    uint32_t q0 = ld(s), q1 = ld(s + 1), q2 = ld(s + 2), q3 = ld(s + 3);
+    for (; s + 4 <= cnt; s += 8) {
+        const uint32_t a0 = q0, a1 = q1, a2 = q2, a3 = q3;
+        q0 = ld(s + 8);
+        q1 = ld(s + 9);
+        q2 = ld(s + 10);
+        q3 = ld(s + 11);
+        body(a0, 0);
+        body(a1, 1);
+        body(a2, 2);
+        body(a3, 3);
     }
-    if (s + 4 <= cnt) {  // four more without a test in between, so that their work overlaps
-#pragma unroll
-        for (int u = 0; u < 4; ++u) body(q[u], u);
-#pragma unroll
-        for (int u = 4; u < 7; ++u)
-            if (s + u < cnt) body(q[u], u);
-    } else {
-#pragma unroll
-        for (int u = 0; u < 3; ++u)
-            if (s + u < cnt) body(q[u], u);
-    }
-}
-
-template <typename real>
-__device__ __forceinline__ real sum8(real a, real b, real c, real d, real e, real f, real g, real h)
-{
-    return ((a + b) + (c + d)) + ((e + f) + (g + h));
+    if (s < cnt) body(q0, 0);
+    if (s + 1 < cnt) body(q1, 1);
+    if (s + 2 < cnt) body(q2, 2);
 }
 
 // 4 consecutive reals (16-byte aligned) into registers
