@@ -458,6 +458,9 @@ int ensure_particles(nep_model* m, int n, int n_items, int n_req, int Tmax)
 
 int ensure_lists(nep_model* m, int n)
 {
+    // no size holds until all of them are there: a call that runs out of memory here leaves
+    // buffers freed, and the next call of any size has to allocate them
+    m->n_lists = 0;
     NEP_TRY(m->nlR.ensure(sizeof(uint32_t) * (size_t)m->mnR * n));
     NEP_TRY(m->nlA.ensure(sizeof(uint32_t) * (size_t)m->mnA * n));
     if (m->precision == NEP_FP64) NEP_TRY(m->fang.ensure(3 * sizeof(double) * (size_t)m->mnA * n));

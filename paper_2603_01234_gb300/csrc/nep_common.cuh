@@ -231,14 +231,12 @@ struct TotalsOut {
     double* all = nullptr;     // [requests][10]: E, W[9]
     double* energy = nullptr;  // [requests]
     double* virial = nullptr;  // [requests][9]
-#ifdef __CUDACC__
     __device__ __forceinline__ void write(int r, int t, double v) const
     {
         all[(size_t)r * 10 + t] = v;
         if (energy && t == 0) energy[r] = v;
         if (virial && t > 0) virial[(size_t)r * 9 + t - 1] = v;
     }
-#endif
 };
 
 template <typename real>

@@ -1,0 +1,115 @@
+"""The library's host code (csrc/capi.cu) on the stand-in CUDA runtime of tests/host_runtime:
+what it allocates, keeps and hands to the kernels, when an allocation fails or a buffer
+moves.  Every array that a kernel would touch is checked against the live allocations."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2603_01234_gb300 import binding, inputs
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def host_library(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("host") / "libnep_host.so")
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-fPIC", "-shared", "-Wl,-Bsymbolic",
+                        "-I", os.path.join(HERE, "host_runtime"), "-I", os.path.join(os.path.dirname(HERE), "include"),
+                        os.path.join(HERE, "host_runtime", "nep_host.cpp"), "-o", out], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return out
+
+
+class Host:
+    def __init__(self, lib):
+        self.lib = lib
+        lib.host_counter.restype = C.c_long
+        lib.host_set.argtypes = [C.c_char_p, C.c_long]
+        lib.host_allocate.restype = C.c_void_p
+        lib.host_allocate.argtypes = [C.c_int, C.c_size_t]
+        for what, value in (("fail_in", -1), ("needR", 20), ("needA", 10)):
+            self.set(what, value)
+        lib.host_reset_counters()
+
+    def set(self, what, value):
+        self.lib.host_set(what.encode(), value)
+
+    def count(self, what):
+        return self.lib.host_counter(what.encode())
+
+    def check(self):
+        """No kernel was given an array that is not there, nor cell counters that are not zero."""
+        assert self.count("bad") == 0 and self.count("uncleared") == 0
+
+
+@pytest.fixture
+def host(host_library, monkeypatch):
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "library_path", lambda: host_library)
+    return Host(binding.load())
+
+
+def model():
+    return inputs.random_model(n_types=1, hidden=5, rc_radial=4.0, rc_angular=3.0, seed=1)
+
+
+def system(n, box=(12.0, 12.0, 12.0)):
+    rng = np.random.default_rng(n)
+    return inputs.System(pos=np.ascontiguousarray(rng.uniform(0, 1, (3, n)) * np.array(box)[:, None]),
+                         types=np.zeros(n, np.int32), box=np.array(box), pbc=np.ones(3, np.int32))
+
+
+def with_failures(host, prepare, call):
+    """Handles on which call() failed at its first, second, ... device allocation, until none is
+    left to fail."""
+    for k in range(200):
+        h = prepare()
+        host.set("fail_in", k)
+        try:
+            call(h)
+            ended = True
+        except binding.NepError as e:
+            assert e.code == binding.NEP_ERR_OOM
+            ended = False
+        host.set("fail_in", -1)
+        yield h
+        host.check()
+        h.close()
+        if ended:
+            return
+    raise AssertionError("allocations without end")
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_lists_after_a_failed_allocation(host, precision):
+    """A call that runs out of memory while it grows the neighbour lists or the pair forces
+    leaves the handle usable: the size that worked before works again, and so does the call."""
+    small, large = system(300), system(6000)
+
+    def prepare():
+        m = binding.Model(model(), precision)
+        m.compute(small)
+        return m
+
+    for m in with_failures(host, prepare, lambda m: m.compute(large)):
+        m.compute(small)
+        m.compute(large)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_lists_after_a_failed_growth(host, precision):
+    """The same when the lists grow because a configuration has more neighbours."""
+    s = system(300)
+
+    def prepare():
+        host.set("needR", 20), host.set("needA", 10)
+        m = binding.Model(model(), precision)
+        m.compute(s)
+        host.set("needR", 500), host.set("needA", 400)
+        return m
+
+    for m in with_failures(host, prepare, lambda m: m.neighbors(s, 0, 4)):
+        m.compute(s)
