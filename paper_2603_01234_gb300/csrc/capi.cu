@@ -231,7 +231,7 @@ struct nep_model {
     Buf partial, partial2, counters, gcounters, totals, flags, thermo, sample_index;
     Buf acc;  // FP32: force and virial fixed-point lines; virial sums for the totals (acc_bytes)
     bool eval_per_bead = false;  // the evaluation in progress returns per-particle virials
-    bool cells_dirty = true;     // the cell counters may be non-zero (a build that failed)
+    bool cells_dirty = true;     // the cell counters may be non-zero (a new buffer, a build that failed)
     Buf types_d, pos_d, vel_d, force_d, virial_d, site_d, force_tmp, totals_tmp;
     Buf noise_d, bussi;  // thermostat: random numbers of the call; [step, alpha] words
     Buf md_virial, md_site, heat, heat_rows;  // HNEMD: per-particle W_i and U_i; acc[6] + counter; rows
@@ -473,16 +473,19 @@ int ensure_cells(nep_model* m, int ncell)
     // the scan leaves the counters of the cells it covers zero for the next build.  A
     // new buffer starts with anything in it and a failed build may leave counts behind,
     // so both are cleared over their whole capacity: a buffer grows by a quarter at
-    // least, and a later grid may reach cells that this one does not.  A new buffer is
-    // told by its capacity: its address may well be the freed one's
-    const size_t c0 = m->cell_count.cap, f0 = m->cell_fill.cap, b0 = m->block_off.cap;
-    NEP_TRY(m->cell_count.ensure(sizeof(int) * ncell));
-    NEP_TRY(m->cell_local.ensure(sizeof(int) * ncell));
-    NEP_TRY(m->block_off.ensure(sizeof(int) * (kScanItems + 1)));
-    NEP_TRY(m->cell_fill.ensure(sizeof(int) * ncell));
-    NEP_TRY(m->cell_start.ensure(sizeof(int) * (ncell + 1)));
-    if (m->cells_dirty || m->cell_count.cap != c0 || m->cell_fill.cap != f0 || m->block_off.cap != b0) {
+    // least, and a later grid may reach cells that this one does not.  What needs
+    // clearing is noted before the first allocation, so that it is still known when a
+    // later one fails and the call ends here
+    auto grows = [](const Buf& b, size_t bytes) { return bytes > b.cap || !b.p; };
+    const size_t bytes = sizeof(int) * (size_t)ncell, scan_bytes = sizeof(int) * (kScanItems + 1);
+    if (grows(m->cell_count, bytes) || grows(m->cell_fill, bytes) || grows(m->block_off, scan_bytes))
         m->cells_dirty = true;
+    NEP_TRY(m->cell_count.ensure(bytes));
+    NEP_TRY(m->cell_local.ensure(bytes));
+    NEP_TRY(m->block_off.ensure(scan_bytes));
+    NEP_TRY(m->cell_fill.ensure(bytes));
+    NEP_TRY(m->cell_start.ensure(sizeof(int) * (ncell + 1)));
+    if (m->cells_dirty) {
         NEP_CUDA(cudaMemsetAsync(m->cell_count.p, 0, m->cell_count.cap, m->cur));
         NEP_CUDA(cudaMemsetAsync(m->cell_fill.p, 0, m->cell_fill.cap, m->cur));
         NEP_CUDA(cudaMemsetAsync(m->block_off.p, 0, m->block_off.cap, m->cur));

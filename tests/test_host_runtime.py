@@ -113,3 +113,19 @@ def test_lists_after_a_failed_growth(host, precision):
 
     for m in with_failures(host, prepare, lambda m: m.neighbors(s, 0, 4)):
         m.compute(s)
+
+
+@pytest.mark.parametrize("later", [(40.0, 40.0, 40.0), (28.0, 28.0, 28.0)])
+def test_cell_counters_after_a_failed_allocation(host, later):
+    """A call that runs out of memory while it grows the cell arrays leaves counters that the
+    next build, of the same grid or of a smaller one, clears before it counts."""
+    first, large, then = system(300), system(300, (40.0, 40.0, 40.0)), system(300, later)
+
+    def prepare():
+        m = binding.Model(model(), "fp32")
+        m.compute(first)
+        return m
+
+    for m in with_failures(host, prepare, lambda m: m.compute(large)):
+        m.compute(then)
+        m.compute(large)
