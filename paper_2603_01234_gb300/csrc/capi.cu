@@ -363,6 +363,7 @@ int upload_plan(nep_model* m, Plan& p, bool force_upload = false)
     put(p.items.data(), sizeof(WorkItem) * p.items.size());
     put(p.models.data(), p.models.size());
     if (!force_upload && key == p.key && p.dev.p) return NEP_OK;
+    p.key.clear();  // until the new tables are on their way (a failure below may leave a new, empty buffer)
     // [counts | models | items | requests]: the items region is laid out by
     // capacity, so the offsets (which the kernels' arguments carry, and a captured
     // graph keeps) depend only on the model count and the item capacity

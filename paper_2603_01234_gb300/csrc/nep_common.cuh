@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <utility>
 
 namespace nep {
@@ -162,7 +163,9 @@ struct ModelDesc {
     const real* params;
     ParamLayout off;
     int T, H;
+    int pad = 0;  // the host compares tables byte by byte: none of them is left to chance
 };
+static_assert(std::has_unique_object_representations_v<ModelDesc<float>>, "padding in a table");
 
 // One request of a batch (device table).
 struct ReqInfo {

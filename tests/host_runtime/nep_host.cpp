@@ -20,8 +20,8 @@ struct Block {
     cudaMemoryType type;
 };
 std::map<char*, Block> blocks;
-size_t device_limit = ~(size_t)0, device_used = 0;
-long fail_in = -1;  // this many more device allocations succeed, then one fails (-1: none)
+// this many more allocations of device (page-locked) memory succeed, then one fails (-1: none)
+long fail_in = -1, fail_host_in = -1;
 int needR = 20, needA = 10;
 std::map<std::string, long> counters;
 
@@ -67,15 +67,11 @@ cudaError_t enqueue(cudaStream_t st, std::function<void()> f)
 cudaError_t allocate(void** p, size_t bytes, cudaMemoryType type)
 {
     const bool dev = type == cudaMemoryTypeDevice;
-    if (dev && (fail_in == 0 || device_used + bytes > device_limit)) {
-        fail_in = fail_in == 0 ? -1 : fail_in;
-        return cudaErrorMemoryAllocation;
-    }
-    if (dev && fail_in > 0) --fail_in;
+    long& f = dev ? fail_in : fail_host_in;
+    if (f >= 0 && f-- == 0) return cudaErrorMemoryAllocation;
     char* q = (char*)aligned_alloc(256, (bytes + 255) / 256 * 256);
     memset(q, 0x5a, bytes);
     blocks[q] = {bytes, type};
-    if (dev) device_used += bytes;
     ++counters[dev ? "malloc" : "malloc_host"];
     *p = q;
     return cudaSuccess;
@@ -85,7 +81,6 @@ cudaError_t release(void* p)
 {
     auto it = blocks.find((char*)p);
     if (it == blocks.end()) return cudaErrorInvalidValue;
-    if (it->second.type == cudaMemoryTypeDevice) device_used -= it->second.bytes;
     blocks.erase(it);
     free(p);
     return cudaSuccess;
@@ -258,7 +253,7 @@ void host_set(const char* what, long value)
 {
     const std::string w = what;
     if (w == "fail_in") fail_in = value;
-    else if (w == "limit") device_limit = (size_t)value;
+    else if (w == "fail_host_in") fail_host_in = value;
     else if (w == "needR") needR = (int)value;
     else if (w == "needA") needA = (int)value;
 }

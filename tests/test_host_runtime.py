@@ -30,7 +30,7 @@ class Host:
         lib.host_set.argtypes = [C.c_char_p, C.c_long]
         lib.host_allocate.restype = C.c_void_p
         lib.host_allocate.argtypes = [C.c_int, C.c_size_t]
-        for what, value in (("fail_in", -1), ("needR", 20), ("needA", 10)):
+        for what, value in (("fail_in", -1), ("fail_host_in", -1), ("needR", 20), ("needA", 10)):
             self.set(what, value)
         lib.host_reset_counters()
 
@@ -129,3 +129,26 @@ def test_cell_counters_after_a_failed_allocation(host, later):
     for m in with_failures(host, prepare, lambda m: m.compute(large)):
         m.compute(then)
         m.compute(large)
+
+
+def batch(m, requests):
+    req_n, box, pbc, types, pos = binding.pack_requests(requests)
+    energy = np.zeros(len(requests))
+    binding.nep_compute_batch([m.h], req_n, np.zeros(len(requests), np.int32), box, pbc, types, pos, energy)
+    return energy
+
+
+def test_plan_tables_after_a_failed_allocation(host):
+    """A batch whose tables get a new device buffer but no staging for their upload leaves no
+    plan that a later call would take for its own."""
+    m = binding.Model(model(), "fp32")
+    small, many = system(300), [system(2)] * 300
+    m.compute(small)
+    host.set("fail_host_in", 0)
+    with pytest.raises(binding.NepError) as e:
+        batch(m, many)
+    assert e.value.code == binding.NEP_ERR_OOM
+    assert m.compute(small)["energy"] == 0.5
+    assert list(batch(m, many)) == [r + 0.5 for r in range(300)]
+    host.check()
+    m.close()
