@@ -160,6 +160,7 @@ struct Plan {
     int n = 0, ncell = 0, n_models = 0;
     int n_cap = 0, items_cap = 0, ncell_cap = 0, req_cap = 0;
     int Tmax = 1;
+    double *energy = nullptr, *virial_total = nullptr;  // where the kernels write the caller's totals (or null)
     size_t smem_desc = 0, smem_force = 0, smem_nbr = 0;
     std::vector<unsigned char> key;     // identity of the uploaded tables
     Buf dev;                            // [counts | reqs | items | models] on the device
@@ -357,7 +358,7 @@ int upload_plan(nep_model* m, Plan& p, bool force_upload = false)
         const unsigned char* b = (const unsigned char*)q;
         key.insert(key.end(), b, b + s);
     };
-    const PlanCounts counts{p.n, (int)p.items.size(), p.ncell, (int)p.reqs.size()};
+    const PlanCounts counts{p.n, (int)p.items.size(), p.ncell, (int)p.reqs.size(), p.energy, p.virial_total};
     put(&counts, sizeof counts);
     put(p.reqs.data(), sizeof(ReqInfo) * p.reqs.size());
     put(p.items.data(), sizeof(WorkItem) * p.items.size());
@@ -402,9 +403,11 @@ const ModelDesc<real>* d_models(const Plan& p)
 }
 
 template <typename real>
-int single_plan(nep_model* m, int n, const CellGrid& g)
+int single_plan(nep_model* m, int n, const CellGrid& g, double* energy = nullptr, double* virial_total = nullptr)
 {
     Plan& p = m->plan;
+    p.energy = energy;
+    p.virial_total = virial_total;
     p.reqs.clear();
     p.items.clear();
     p.n = p.ncell = 0;
@@ -611,7 +614,7 @@ struct FusedKick {
 };
 
 template <typename real>
-int run_evaluate(nep_model* m, const Plan& p, double* force, double* virial, double* site, const TotalsOut& totals,
+int run_evaluate(nep_model* m, const Plan& p, double* force, double* virial, double* site, double* totals,
                  cudaEvent_t mid = nullptr, const FusedKick* kick = nullptr)
 {
     EvalArgs<real> a;
@@ -692,7 +695,7 @@ int check_lists(nep_model* m, const Plan& p)
 // force must be non-null.
 template <typename real>
 int evaluate_plan(nep_model* m, const Plan& p, const int* types_d, const double* pos_d, double* force,
-                  double* virial, double* site, const TotalsOut& totals)
+                  double* virial, double* site, double* totals)
 {
     NEP_TRY(ensure_plan_workspace(m, p));
     m->eval_per_bead = virial != nullptr;
@@ -710,7 +713,7 @@ int evaluate_plan(nep_model* m, const Plan& p, const int* types_d, const double*
 // from them after the call synchronised (eval_status).
 template <typename real>
 int eval_pipeline(nep_model* m, const Plan& p, const int* types_d, const double* pos_d, double* force,
-                  double* virial, double* site, const TotalsOut& totals)
+                  double* virial, double* site, double* totals)
 {
     NEP_CUDA(cudaMemsetAsync(m->flags.p, 0, 3 * sizeof(int), m->cur));
     NEP_TRY(run_cells<real>(m, p, types_d, pos_d));
@@ -763,12 +766,12 @@ std::vector<unsigned char> eval_graph_key(const nep_model* m, const Plan& p, con
 // similar size share one graph.
 template <typename real>
 int eval_launch(nep_model* m, const Plan& p, const int* types_d, const double* pos_d, double* force,
-                double* virial, double* site, const TotalsOut& totals)
+                double* virial, double* site, double* totals)
 {
     NEP_TRY(ensure_plan_workspace(m, p));
     m->eval_per_bead = virial != nullptr;
-    const void* io[] = {types_d, pos_d, force, virial, site, totals.all, totals.energy, totals.virial};
-    std::vector<unsigned char> key = eval_graph_key<real>(m, p, io, 8);
+    const void* io[] = {types_d, pos_d, force, virial, site, totals};
+    std::vector<unsigned char> key = eval_graph_key<real>(m, p, io, 6);
     for (size_t k = 0; k < m->eval_graphs.size(); ++k)
         if (m->eval_graphs[k].key == key) {
             NEP_CUDA(cudaGraphLaunch(m->eval_graphs[k].exec, m->cur));
@@ -895,12 +898,13 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
     NEP_TRY(make_grid(m, box, pbc, g));
     NEP_TRY(enter(m, stream));
     initial_capacity(m, n, box);
-    NEP_TRY(single_plan<real>(m, n, g));
+    if (mem == NEP_DEVICE) NEP_TRY(single_plan<real>(m, n, g, energy_total, virial_total));
+    else NEP_TRY(single_plan<real>(m, n, g));
     NEP_TRY(ensure_plan_workspace(m, m->plan));
     const int* types_d = types;
     const double* pos_d = pos;
     double *force_d = force, *virial_d = virial, *site_d = site_energy;
-    TotalsOut totals{m->totals.as<double>(), energy_total, virial_total};
+    double* totals = m->totals.as<double>();
     double* out = nullptr;  // a small host call's outputs in pinned memory: totals, force, virial, site energies
     if (mem == NEP_HOST && n <= kDirectMaxN) {
         // the kernels read the inputs and write the outputs in page-locked memory, each
@@ -913,13 +917,12 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
         memcpy(in + 3 * (size_t)n, types, sizeof(int) * (size_t)n);
         pos_d = in;
         types_d = (const int*)(in + 3 * (size_t)n);
-        totals = TotalsOut{out};
+        totals = out;
         force_d = out + 10;
         virial_d = virial ? out + 10 + 3 * (size_t)n : nullptr;
         site_d = site_energy ? out + 10 + 12 * (size_t)n : nullptr;
     } else if (mem == NEP_HOST) {
         NEP_TRY(ensure_host_totals(m, 10));
-        totals = TotalsOut{m->totals.as<double>()};
         NEP_TRY(m->types_d.ensure(sizeof(int) * n));
         NEP_TRY(m->pos_d.ensure(sizeof(double) * 3 * (size_t)n));
         NEP_CUDA(cudaMemcpyAsync(m->types_d.p, types, sizeof(int) * n, cudaMemcpyHostToDevice, m->cur));
@@ -951,7 +954,7 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
                 NEP_CUDA(cudaMemcpyAsync(virial, virial_d, sizeof(double) * 9 * n, cudaMemcpyDeviceToHost, m->cur));
             if (site_energy)
                 NEP_CUDA(cudaMemcpyAsync(site_energy, site_d, sizeof(double) * n, cudaMemcpyDeviceToHost, m->cur));
-            NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals.all, sizeof(double) * 10, cudaMemcpyDeviceToHost, m->cur));
+            NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals, sizeof(double) * 10, cudaMemcpyDeviceToHost, m->cur));
         }
         NEP_TRY(leave(m, stream));
         bool retry = false;
@@ -1019,7 +1022,7 @@ int autotune_plan(nep_model* m, const Plan& p, double* force_d)
         m->mb_force = t.mf;
         m->ch_force = t.ch;
         NEP_CUDA(cudaEventRecord(e0, m->cur));
-        NEP_TRY(run_evaluate<real>(m, p, force_d, nullptr, nullptr, TotalsOut{m->totals.as<double>()}, em));
+        NEP_TRY(run_evaluate<real>(m, p, force_d, nullptr, nullptr, m->totals.as<double>(), em));
         NEP_CUDA(cudaEventRecord(e1, m->cur));
         NEP_CUDA(cudaEventSynchronize(e1));
         if (!timed) return NEP_OK;
@@ -1078,7 +1081,7 @@ int md_forces(nep_model* m, const Plan& p, int n, double* force, const Drive& dr
 {
     if (kick && dr.on) return fail(NEP_ERR_ARG, "the driving force precedes the closing kick");
     NEP_TRY(run_evaluate<real>(m, p, force, dr.on ? dr.virial : nullptr, dr.on ? dr.site : nullptr,
-                               TotalsOut{m->totals.as<double>()}, mid, kick));
+                               m->totals.as<double>(), mid, kick));
     if (dr.on) {
         cudaError_t e = launch_hnemd_force(n, dr.fe, dr.virial, m->totals.as<double>(), force, m->cur);
         if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("driving force: ") + cudaGetErrorString(e));
@@ -1497,6 +1500,8 @@ int batch_impl(nep_model* const* models, int n_models, int n_req, const int32_t*
             return fail(NEP_ERR_ARG, "batch cell grids too large");
         add_request(p, g, req_n[r], req_model[r]);
     }
+    p.energy = mem == NEP_DEVICE ? energy : nullptr;
+    p.virial_total = mem == NEP_DEVICE ? virial_total : nullptr;
     set_caps(p, true);  // size classes: batches of similar size replay one graph
     set_models<real>(p, models, n_models);
     (void)rc_max;
@@ -1536,11 +1541,7 @@ int batch_impl(nep_model* const* models, int n_models, int n_req, const int32_t*
     } else if (!force_d) {
         force_d = m->force_tmp.as<double>();
     }
-    TotalsOut totals{m->totals.as<double>()};
-    if (mem == NEP_DEVICE) {
-        totals.energy = energy;
-        totals.virial = virial_total;
-    }
+    double* totals = m->totals.as<double>();
     NEP_TRY(ensure_host_totals(m, 10 * (size_t)n_req));
     // one synchronisation per batch (see compute_impl)
     for (int attempt = 0;; ++attempt) {
@@ -1551,7 +1552,7 @@ int batch_impl(nep_model* const* models, int n_models, int n_req, const int32_t*
                 NEP_CUDA(cudaMemcpyAsync(virial, virial_d, sizeof(double) * 9 * n, cudaMemcpyDeviceToHost, m->cur));
             if (site_energy)
                 NEP_CUDA(cudaMemcpyAsync(site_energy, site_d, sizeof(double) * n, cudaMemcpyDeviceToHost, m->cur));
-            NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals.all, sizeof(double) * 10 * n_req, cudaMemcpyDeviceToHost,
+            NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals, sizeof(double) * 10 * n_req, cudaMemcpyDeviceToHost,
                                      m->cur));
         }
         NEP_TRY(leave(m, stream));
@@ -2062,12 +2063,12 @@ int nep_autotune(nep_model* m, int n, const int32_t* types, const double* pos, c
         rc = single_plan<double>(m, n, g);
         if (rc == NEP_OK) rc = ensure_plan_workspace(m, m->plan);
         if (rc == NEP_OK) rc = evaluate_plan<double>(m, m->plan, types_d, pos_d, m->force_tmp.as<double>(), nullptr,
-                                                     nullptr, TotalsOut{m->totals.as<double>()});
+                                                     nullptr, m->totals.as<double>());
     } else {
         rc = single_plan<float>(m, n, g);
         if (rc == NEP_OK) rc = ensure_plan_workspace(m, m->plan);
         if (rc == NEP_OK) rc = evaluate_plan<float>(m, m->plan, types_d, pos_d, m->force_tmp.as<double>(), nullptr,
-                                                    nullptr, TotalsOut{m->totals.as<double>()});
+                                                    nullptr, m->totals.as<double>());
         if (rc == NEP_OK) rc = autotune_plan<float>(m, m->plan, m->force_tmp.as<double>());
     }
     NEP_TRY(rc);
@@ -2375,7 +2376,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     for (int b = 0; b < n; b += kBlock) items[n_items++] = WorkItem{0, b, std::min(n, b + kBlock)};
     rq.item_end = n_items;
     const ModelDesc<real> md = model_desc<real>(m);
-    const PlanCounts counts{n, n_items, g.ncell, 1};
+    const PlanCounts counts{n, n_items, g.ncell, 1, energy_total, virial_total};
     const size_t off_rq = align16(sizeof(PlanCounts)), off_items = off_rq + align16(sizeof(ReqInfo)),
                  off_models = off_items + align16(sizeof(WorkItem) * n_items);
     if (m->plan_pending) NEP_CUDA(cudaEventSynchronize(m->ev_plan));
@@ -2457,7 +2458,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     a.gcounter = counters + 1;  // one group: at most kStaticMaxN / 128 <= 32 work items
     a.icounter = counters + 4;
     a.err = flags + 2;
-    a.totals = TotalsOut{totals, energy_total, virial_total};
+    a.totals = totals;
     e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, n_items, m->smem_desc, m->smem_force, m->cur, nullptr,
                               m->mb_desc, m->mb_force, m->ch_force);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("evaluate: ") + cudaGetErrorString(e));

@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kBlock, MB) k_force_radial(EvalArgs<real> a)
 #pragma unroll
         for (int k = 0; k < 9; ++k) tot[1 + k] = (double)(a.wsum[(size_t)k * a.n + i] + Wr[k]);
     }
-    reduce_totals<kBlock>(tot, w, it, rq, a.partial, a.gcounter, a.counter, a.totals);
+    reduce_totals<kBlock>(tot, w, it, rq, a.partial, a.gcounter, a.counter, a.counts, a.totals);
 }
 
 // ---- shape dispatch -----------------------------------------------------------

@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
 #pragma unroll
         for (int k = 0; k < 9; ++k) tot[1 + k] = (double)__ldcg(a.wsum + (size_t)k * n + it_i);
     }
-    reduce_totals<kBlock>(tot, item, it, rq, a.partial, a.gcounter, a.counter, a.totals);
+    reduce_totals<kBlock>(tot, item, it, rq, a.partial, a.gcounter, a.counter, a.counts, a.totals);
 }
 
 template <typename real, int NA>

@@ -622,7 +622,7 @@ __device__ __forceinline__ double sum_partials(const double* src, int nb, int st
 template <int BS>
 __device__ __forceinline__ void reduce_totals(double (&v)[10], int item, const WorkItem& it, const ReqInfo& rq,
                                               double* partial, unsigned int* gcounter, unsigned int* counter,
-                                              const TotalsOut& out)
+                                              const PlanCounts* counts, double* totals)
 {
     static_assert(BS % 8 == 0 && BS >= 120, "block size");
     __shared__ double red[10][BS + 8];  // row stride 2 words mod 32 apart: 2-way for 64-bit loads
@@ -659,7 +659,7 @@ __device__ __forceinline__ void reduce_totals(double (&v)[10], int item, const W
     const double gs = sum_partials(partial + (size_t)g0 * 10, gn, 1, part);
     const int ng = (n_items + kGroup - 1) / kGroup;
     if (ng == 1) {  // one group: its sum is the total
-        if (t < 10) out.write(it.req, t, gs);
+        if (t < 10) write_total(*counts, totals, it.req, t, gs);
         if (t == 0) gcounter[g0] = 0u;
         return;
     }
@@ -674,7 +674,7 @@ __device__ __forceinline__ void reduce_totals(double (&v)[10], int item, const W
     if (!last) return;
     __threadfence();
     const double ts = sum_partials(partial + (size_t)rq.item_begin * 10, ng, kGroup, part);
-    if (t < 10) out.write(it.req, t, ts);
+    if (t < 10) write_total(*counts, totals, it.req, t, ts);
     if (t == 0) counter[it.req] = 0u;
 }
 

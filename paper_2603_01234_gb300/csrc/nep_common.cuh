@@ -181,12 +181,15 @@ struct WorkItem {
     int req, begin, end;
 };
 
-// Sizes of the batch in progress, in device memory ahead of its tables.  The
-// kernels take their loop bounds from here and loop over work items with a grid
-// stride, so launch shapes depend only on capacities: one captured CUDA graph then
-// serves every batch that fits them.
+// Sizes of the batch in progress, in device memory ahead of its tables, and the caller's own
+// arrays for the totals (either may be null).  The kernels take their bounds from here, so
+// launch shapes depend only on capacities, and the totals' addresses, which a program may
+// change from call to call (each frame's energy into the next place of an array): one captured
+// CUDA graph then serves every batch that fits it.
 struct PlanCounts {
     int n, n_items, ncell, n_req;
+    double* energy;  // [requests]
+    double* virial;  // [requests][9]
 };
 
 template <typename real>
@@ -228,19 +231,13 @@ constexpr int kGroup = 32;
 // touching memory out of bounds.
 constexpr int kErrCellList = 4;
 
-// Where the totals of request r go: all ten together, and the caller's own arrays (either may
-// be absent).
-struct TotalsOut {
-    double* all = nullptr;     // [requests][10]: E, W[9]
-    double* energy = nullptr;  // [requests]
-    double* virial = nullptr;  // [requests][9]
-    __device__ __forceinline__ void write(int r, int t, double v) const
-    {
-        all[(size_t)r * 10 + t] = v;
-        if (energy && t == 0) energy[r] = v;
-        if (virial && t > 0) virial[(size_t)r * 9 + t - 1] = v;
-    }
-};
+// Total t (E, then W[9]) of request r: into all [requests][10] and the caller's own arrays.
+__device__ __forceinline__ void write_total(const PlanCounts& pc, double* all, int r, int t, double v)
+{
+    all[(size_t)r * 10 + t] = v;
+    if (pc.energy && t == 0) pc.energy[r] = v;
+    if (pc.virial && t > 0) pc.virial[(size_t)r * 9 + t - 1] = v;
+}
 
 template <typename real>
 struct EvalArgs {
@@ -275,7 +272,7 @@ struct EvalArgs {
     unsigned int* gcounter;     // [items] last-block counters of the item groups, at each
                                 // group's first item (self-resetting)
     unsigned int* icounter;     // [items] group kernels: finished blocks of each item (self-resetting)
-    TotalsOut totals;           // per request: E, W[9]
+    double* totals;             // [requests][10]: E, W[9]
     int* err = nullptr;         // the error word (kErrCellList on an inconsistent cell list)
     // MD: the step's closing half-kick applied by the output pass as soon as F_i is
     // final, v_i <- half_kick(v_i, kick_half_dt, F_i, kick_im[t_i]), with the same

@@ -11,6 +11,17 @@
 #include <string>
 #include <vector>
 
+#include <cuda_runtime.h>
+
+void host_symbol(void* p, size_t bytes);
+template <typename T>
+cudaError_t cudaGetSymbolAddress(void** p, T& symbol)
+{
+    *p = (void*)&symbol;
+    host_symbol(*p, sizeof symbol);
+    return cudaSuccess;
+}
+
 #include "../../paper_2603_01234_gb300/csrc/capi.cu"
 
 namespace {
@@ -88,6 +99,7 @@ cudaError_t release(void* p)
 
 }  // namespace
 
+void host_symbol(void* p, size_t bytes) { blocks[(char*)p] = {bytes, cudaMemoryTypeDevice}; }
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaErrorMemoryAllocation ? "out of memory" : "error"; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
@@ -145,7 +157,7 @@ int neighbor_form(int, int, int, bool) { return 1; }
 bool evaluate_by_groups(int, bool) { return true; }
 
 template <typename real>
-cudaError_t launch_cell_build(const PlanCounts*, int n_cap, int, int ncell_cap, bool zero_counts, bool, const WorkItem*,
+cudaError_t launch_cell_build(const PlanCounts* pc, int n_cap, int, int ncell_cap, bool zero_counts, bool, const WorkItem*,
                               const ReqInfo*, const ModelDesc<real>*, const double* pos, const int* types, int* cell_of,
                               PosRec<real>* rec_user, int* cell_count, int* cell_local, int* block_off, int* cell_fill,
                               int* perm_tmp, int* perm, int* cell_start, int* cell_s, PosRec<real>* rec_s, int* err,
@@ -153,7 +165,7 @@ cudaError_t launch_cell_build(const PlanCounts*, int n_cap, int, int ncell_cap, 
 {
     return enqueue(st, [=] {
         const size_t n = n_cap, nc = ncell_cap;
-        reach("pos", pos, 8 * n), reach("types", types, 4 * n), reach("cell_of", cell_of, 4 * n);
+        reach("pos", pos, 24 * (size_t)pc->n), reach("types", types, 4 * (size_t)pc->n), reach("cell_of", cell_of, 4 * n);
         reach("rec", rec_user, sizeof(PosRec<real>) * n), reach("rec_s", rec_s, sizeof(PosRec<real>) * n);
         reach("perm", perm, 4 * n), reach("perm_tmp", perm_tmp, 4 * n), reach("cell_s", cell_s, 4 * n);
         reach("cell_local", cell_local, 4 * nc), reach("cell_fill", cell_fill, 4 * nc), reach("cell_start", cell_start, 4 * (nc + 1));
@@ -207,12 +219,12 @@ cudaError_t launch_evaluate(int, int, int, int, const EvalArgs<real>& a, int ite
         if (sizeof(real) == 8) reach("fang", a.fang, 24 * n * a.mnA);
         else reach("accF", a.accF, 32 * n);
         const size_t nq = a.counts->n_req;
-        reach("totals", a.totals.all, 80 * nq);
-        if (a.totals.energy) reach("energy", a.totals.energy, 8 * nq);
-        if (a.totals.virial) reach("virial_total", a.totals.virial, 72 * nq);
+        reach("totals", a.totals, 80 * nq);
+        if (a.counts->energy) reach("energy", a.counts->energy, 8 * nq);
+        if (a.counts->virial) reach("virial_total", a.counts->virial, 72 * nq);
         if (counters["bad"]) return;
         for (size_t r = 0; r < nq; ++r)  // energy r + 0.5, virial component k r + k
-            for (int t = 0; t < 10; ++t) a.totals.write((int)r, t, (double)r + (t ? t - 1 : 0.5));
+            for (int t = 0; t < 10; ++t) write_total(*a.counts, a.totals, (int)r, t, (double)r + (t ? t - 1 : 0.5));
     });
 }
 

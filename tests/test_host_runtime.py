@@ -152,3 +152,57 @@ def test_plan_tables_after_a_failed_allocation(host):
     assert list(batch(m, many)) == [r + 0.5 for r in range(300)]
     host.check()
     m.close()
+
+
+class DeviceCall:
+    """nep_compute (or its variants) on arrays of the stand-in device, one configuration."""
+
+    def __init__(self, host, m, s):
+        self.m, self.s, self.host = m, s, host
+        self.types, self.pos = self.device(s.types), self.device(s.pos)
+        self.force = self.device(np.zeros((3, s.n)))
+
+    def device(self, a):
+        p = self.host.lib.host_allocate(2, a.nbytes)
+        C.memmove(p, a.ctypes.data, a.nbytes)
+        return p
+
+    def __call__(self, name, energy, virial):
+        lib, s, ptr = self.host.lib, self.s, binding._ptr
+        one = (self.types, self.pos, ptr(s.box), ptr(s.pbc))
+        out = (energy, virial, None, self.force, None)
+        if name == "batch":  # two requests of the one configuration's halves
+            n = np.array([s.n // 2, s.n - s.n // 2], np.int32)
+            box, pbc = np.tile(s.box, 2), np.tile(s.pbc, 2)
+            h, which = (C.c_void_p * 1)(self.m.h), np.zeros(2, np.int32)
+            rc = lib.nep_compute_batch(C.cast(h, C.c_void_p), 1, 2, ptr(n), ptr(which), ptr(box), ptr(pbc), self.types,
+                                       self.pos, binding.NEP_DEVICE, None, *out)
+        elif name == "static":
+            rc = lib.nep_compute_static(self.m.h, s.n, *one, None, *out)
+        else:
+            rc = lib.nep_compute(self.m.h, s.n, *one, binding.NEP_DEVICE, None, *out)
+        binding._check(rc, name)
+
+
+def doubles(address, count):
+    return list(np.frombuffer(C.string_at(address, 8 * count)))
+
+
+@pytest.mark.parametrize("name,requests", [("compute", 1), ("batch", 2), ("static", 1)])
+def test_totals_at_other_addresses_replay_one_graph(host, name, requests):
+    """A program that takes each frame's totals into another place, its other arrays staying
+    where they are, replays one captured graph."""
+    m = binding.Model(model(), "fp32")
+    call = DeviceCall(host, m, system(300))
+    E, W = call.device(np.zeros(2 * 40)), call.device(np.zeros(18 * 40))
+    for k in range(200):
+        at = k % 40
+        e, w = E + 16 * at, W + 144 * at
+        C.memset(e, 0, 8 * requests), C.memset(w, 0, 72 * requests)
+        call(name, e, w)
+        assert doubles(e, requests) == [0.5, 1.5][:requests]
+        assert doubles(w, 9 * requests) == [float(r + c) for r in range(requests) for c in range(9)]
+        if name != "static":  # launched once by itself and once into the graph
+            assert host.count("evaluate") == min(k, 1) + 1 and host.count("instantiate") == min(k, 1)
+    host.check()
+    m.close()
