@@ -873,6 +873,40 @@ int ensure_host_totals(nep_model* m, size_t count)
     return NEP_OK;
 }
 
+// An array of the caller's for totals: the kernels write it where they can (aligned, in memory
+// that this device reaches); elsewhere (a field of a packed record, another device) it gets
+// a copy, which takes any address.
+struct TotalsTarget {
+    double *direct = nullptr, *copied = nullptr;
+};
+
+TotalsTarget totals_target(const nep_model* m, double* p)
+{
+    TotalsTarget t;
+    if (!p) return t;
+    cudaPointerAttributes a;
+    bool reached = (uintptr_t)p % alignof(double) == 0;
+    if (reached && cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        reached = false;
+    }
+    reached = reached && (a.type == cudaMemoryTypeDevice ? a.device == m->device : a.type != cudaMemoryTypeUnregistered);
+    (reached ? t.direct : t.copied) = p;
+    return t;
+}
+
+// The totals [n_req][10] into arrays that get copies.
+int copy_totals(nep_model* m, const double* totals, size_t n_req, const TotalsTarget& energy, const TotalsTarget& virial)
+{
+    auto part = [&](double* to, const double* from, size_t words) {
+        return cudaMemcpy2DAsync(to, words * sizeof(double), from, 10 * sizeof(double), words * sizeof(double), n_req,
+                                 cudaMemcpyDeviceToDevice, m->cur);
+    };
+    if (energy.copied) NEP_CUDA(part(energy.copied, totals, 1));
+    if (virial.copied) NEP_CUDA(part(virial.copied, totals + 1, 9));
+    return NEP_OK;
+}
+
 // Particles up to which a host call works on page-locked memory directly.  Measured (water,
 // FP32, whole call): 64 particles 96 us against 127 with copies, 1,000 108 / 136, 4,000
 // 148 / 166; the buffer stays below 0.6 MB.
@@ -898,8 +932,12 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
     NEP_TRY(make_grid(m, box, pbc, g));
     NEP_TRY(enter(m, stream));
     initial_capacity(m, n, box);
-    if (mem == NEP_DEVICE) NEP_TRY(single_plan<real>(m, n, g, energy_total, virial_total));
-    else NEP_TRY(single_plan<real>(m, n, g));
+    TotalsTarget to_energy, to_virial;
+    if (mem == NEP_DEVICE) {
+        to_energy = totals_target(m, energy_total);
+        to_virial = totals_target(m, virial_total);
+    }
+    NEP_TRY(single_plan<real>(m, n, g, to_energy.direct, to_virial.direct));
     NEP_TRY(ensure_plan_workspace(m, m->plan));
     const int* types_d = types;
     const double* pos_d = pos;
@@ -956,6 +994,7 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
                 NEP_CUDA(cudaMemcpyAsync(site_energy, site_d, sizeof(double) * n, cudaMemcpyDeviceToHost, m->cur));
             NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals, sizeof(double) * 10, cudaMemcpyDeviceToHost, m->cur));
         }
+        NEP_TRY(copy_totals(m, totals, 1, to_energy, to_virial));
         NEP_TRY(leave(m, stream));
         bool retry = false;
         NEP_TRY(eval_status(m, retry));
@@ -1500,8 +1539,13 @@ int batch_impl(nep_model* const* models, int n_models, int n_req, const int32_t*
             return fail(NEP_ERR_ARG, "batch cell grids too large");
         add_request(p, g, req_n[r], req_model[r]);
     }
-    p.energy = mem == NEP_DEVICE ? energy : nullptr;
-    p.virial_total = mem == NEP_DEVICE ? virial_total : nullptr;
+    TotalsTarget to_energy, to_virial;
+    if (mem == NEP_DEVICE) {
+        to_energy = totals_target(m, energy);
+        to_virial = totals_target(m, virial_total);
+    }
+    p.energy = to_energy.direct;
+    p.virial_total = to_virial.direct;
     set_caps(p, true);  // size classes: batches of similar size replay one graph
     set_models<real>(p, models, n_models);
     (void)rc_max;
@@ -1555,6 +1599,7 @@ int batch_impl(nep_model* const* models, int n_models, int n_req, const int32_t*
             NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals, sizeof(double) * 10 * n_req, cudaMemcpyDeviceToHost,
                                      m->cur));
         }
+        NEP_TRY(copy_totals(m, totals, n_req, to_energy, to_virial));
         NEP_TRY(leave(m, stream));
         bool retry = false;
         NEP_TRY(eval_status(m, retry));
@@ -2376,7 +2421,8 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     for (int b = 0; b < n; b += kBlock) items[n_items++] = WorkItem{0, b, std::min(n, b + kBlock)};
     rq.item_end = n_items;
     const ModelDesc<real> md = model_desc<real>(m);
-    const PlanCounts counts{n, n_items, g.ncell, 1, energy_total, virial_total};
+    const TotalsTarget to_energy = totals_target(m, energy_total), to_virial = totals_target(m, virial_total);
+    const PlanCounts counts{n, n_items, g.ncell, 1, to_energy.direct, to_virial.direct};
     const size_t off_rq = align16(sizeof(PlanCounts)), off_items = off_rq + align16(sizeof(ReqInfo)),
                  off_models = off_items + align16(sizeof(WorkItem) * n_items);
     if (m->plan_pending) NEP_CUDA(cudaEventSynchronize(m->ev_plan));
@@ -2462,6 +2508,7 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, n_items, m->smem_desc, m->smem_force, m->cur, nullptr,
                               m->mb_desc, m->mb_force, m->ch_force);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("evaluate: ") + cudaGetErrorString(e));
+    NEP_TRY(copy_totals(m, totals, 1, to_energy, to_virial));
     // the handle's pinned status buffer (allocated by nep_create) receives the words
     NEP_CUDA(cudaMemcpyAsync(m->h_flags, flags, 3 * sizeof(int), cudaMemcpyDeviceToHost, m->cur));
     NEP_CUDA(cudaStreamSynchronize(m->cur));

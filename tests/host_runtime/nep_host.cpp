@@ -29,6 +29,7 @@ namespace {
 struct Block {
     size_t bytes;
     cudaMemoryType type;
+    int device = 0;
 };
 std::map<char*, Block> blocks;
 // this many more allocations of device (page-locked) memory succeed, then one fails (-1: none)
@@ -48,7 +49,7 @@ const std::pair<char* const, Block>* block_of(const void* p)
 void reach(const char* what, const void* p, size_t bytes)
 {
     const auto* b = p ? block_of(p) : nullptr;
-    if (b && (const char*)p + bytes <= b->first + b->second.bytes && b->second.type != cudaMemoryTypeUnregistered) return;
+    if (b && (const char*)p + bytes <= b->first + b->second.bytes && b->second.device == 0) return;
     ++counters["bad"];
     ++counters[std::string("bad ") + what];
 }
@@ -112,7 +113,7 @@ cudaError_t cudaFreeHost(void* p) { return release(p); }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p)
 {
     const auto* b = block_of(p);
-    *a = {b ? b->second.type : cudaMemoryTypeUnregistered, 0, (void*)p, (void*)p};
+    *a = {b ? b->second.type : cudaMemoryTypeUnregistered, b ? b->second.device : -1, (void*)p, (void*)p};
     return cudaSuccess;
 }
 cudaError_t cudaMemset(void* p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
@@ -122,6 +123,10 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cu
 {
     ++counters["copies"];
     return enqueue(st, [=] { memcpy(d, s, n); });
+}
+cudaError_t cudaMemcpy2DAsync(void* d, size_t dp, const void* s, size_t sp, size_t w, size_t h, cudaMemcpyKind, cudaStream_t st)
+{
+    return enqueue(st, [=] { for (size_t k = 0; k < h; ++k) memcpy((char*)d + k * dp, (const char*)s + k * sp, w); });
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = new HostStream; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { delete s; return cudaSuccess; }
@@ -222,6 +227,7 @@ cudaError_t launch_evaluate(int, int, int, int, const EvalArgs<real>& a, int ite
         reach("totals", a.totals, 80 * nq);
         if (a.counts->energy) reach("energy", a.counts->energy, 8 * nq);
         if (a.counts->virial) reach("virial_total", a.counts->virial, 72 * nq);
+        if ((uintptr_t)a.counts->energy % 8 || (uintptr_t)a.counts->virial % 8) ++counters["bad"];
         if (counters["bad"]) return;
         for (size_t r = 0; r < nq; ++r)  // energy r + 0.5, virial component k r + k
             for (int t = 0; t < 10; ++t) write_total(*a.counts, a.totals, (int)r, t, (double)r + (t ? t - 1 : 0.5));
@@ -269,11 +275,14 @@ void host_set(const char* what, long value)
     else if (w == "needR") needR = (int)value;
     else if (w == "needA") needA = (int)value;
 }
-// memory of the stand-in device (kind 2) or page-locked memory (1)
+// memory of the stand-in device (kind 2), of another device that kernels do not reach (3), or
+// page-locked memory (1)
 void* host_allocate(int kind, size_t bytes)
 {
     void* p = nullptr;
-    return (kind == 2 ? cudaMalloc(&p, bytes) : cudaMallocHost(&p, bytes)) == cudaSuccess ? p : nullptr;
+    if ((kind == 1 ? cudaMallocHost(&p, bytes) : cudaMalloc(&p, bytes)) != cudaSuccess) return nullptr;
+    if (kind == 3) blocks[(char*)p].device = 1;
+    return p;
 }
 long host_counter(const char* what) { return counters[what]; }
 void host_reset_counters() { counters.clear(); }

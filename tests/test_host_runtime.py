@@ -206,3 +206,21 @@ def test_totals_at_other_addresses_replay_one_graph(host, name, requests):
             assert host.count("evaluate") == min(k, 1) + 1 and host.count("instantiate") == min(k, 1)
     host.check()
     m.close()
+
+
+@pytest.mark.parametrize("where", ["unaligned", "other_device", "page_locked"])
+@pytest.mark.parametrize("name,requests", [("compute", 1), ("batch", 2), ("static", 1)])
+def test_totals_where_the_kernels_cannot_write(host, name, requests, where):
+    """Totals at an address that is no multiple of eight bytes, or on a device that the kernels do
+    not reach, arrive by a copy; no kernel gets such an address."""
+    m = binding.Model(model(), "fp32")
+    call = DeviceCall(host, m, system(300))
+    kind = {"unaligned": 2, "other_device": 3, "page_locked": 1}[where]
+    e, w = (host.lib.host_allocate(kind, 1024) + (4 if where == "unaligned" else 0) for _ in range(2))
+    for k in range(3):
+        C.memset(e, 0, 8 * requests), C.memset(w, 0, 72 * requests)
+        call(name, e, w)
+        assert doubles(e, requests) == [0.5, 1.5][:requests]
+        assert doubles(w, 9 * requests) == [float(r + c) for r in range(requests) for c in range(9)]
+    host.check()
+    m.close()
