@@ -912,6 +912,18 @@ int copy_totals(nep_model* m, const double* totals, size_t n_req, const TotalsTa
 // 148 / 166; the buffer stays below 0.6 MB.
 constexpr int kDirectMaxN = 4096;
 
+// Whether the CPU may read and write p: device memory among the arrays of a host call takes the
+// copies, which reach it.
+bool cpu_reaches(const void* p)
+{
+    cudaPointerAttributes a;
+    if (p && cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return !p || a.type != cudaMemoryTypeDevice;
+}
+
 int ensure_host_io(nep_model* m, size_t bytes)
 {
     if (bytes <= m->h_io_cap) return NEP_OK;
@@ -944,7 +956,8 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
     double *force_d = force, *virial_d = virial, *site_d = site_energy;
     double* totals = m->totals.as<double>();
     double* out = nullptr;  // a small host call's outputs in pinned memory: totals, force, virial, site energies
-    if (mem == NEP_HOST && n <= kDirectMaxN) {
+    if (mem == NEP_HOST && n <= kDirectMaxN && cpu_reaches(types) && cpu_reaches(pos) && cpu_reaches(force) &&
+        cpu_reaches(virial) && cpu_reaches(site_energy)) {
         // the kernels read the inputs and write the outputs in page-locked memory, each
         // value once: no copies, whose launches would take longer than the transfers
         const size_t words = 10 + 13 * (size_t)n + 3 * (size_t)n;  // doubles, then n ints

@@ -36,6 +36,7 @@ std::map<char*, Block> blocks;
 long fail_in = -1, fail_host_in = -1;
 int needR = 20, needA = 10;
 std::map<std::string, long> counters;
+std::map<const void*, long> copies;  // by their addresses
 
 const std::pair<char* const, Block>* block_of(const void* p)
 {
@@ -121,7 +122,8 @@ cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t st) { return 
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st)
 {
-    ++counters["copies"];
+    ++copies[d];
+    ++copies[s];
     return enqueue(st, [=] { memcpy(d, s, n); });
 }
 cudaError_t cudaMemcpy2DAsync(void* d, size_t dp, const void* s, size_t sp, size_t w, size_t h, cudaMemcpyKind, cudaStream_t st)
@@ -285,5 +287,6 @@ void* host_allocate(int kind, size_t bytes)
     return p;
 }
 long host_counter(const char* what) { return counters[what]; }
+long host_copies(const void* p) { return copies[p]; }
 void host_reset_counters() { counters.clear(); }
 }

@@ -30,6 +30,8 @@ class Host:
         lib.host_set.argtypes = [C.c_char_p, C.c_long]
         lib.host_allocate.restype = C.c_void_p
         lib.host_allocate.argtypes = [C.c_int, C.c_size_t]
+        lib.host_copies.restype = C.c_long
+        lib.host_copies.argtypes = [C.c_void_p]
         for what, value in (("fail_in", -1), ("fail_host_in", -1), ("needR", 20), ("needA", 10)):
             self.set(what, value)
         lib.host_reset_counters()
@@ -222,5 +224,24 @@ def test_totals_where_the_kernels_cannot_write(host, name, requests, where):
         call(name, e, w)
         assert doubles(e, requests) == [0.5, 1.5][:requests]
         assert doubles(w, 9 * requests) == [float(r + c) for r in range(requests) for c in range(9)]
+    host.check()
+    m.close()
+
+
+def test_small_host_calls_with_device_memory_among_their_arrays(host):
+    """A small host call works on page-locked memory that the CPU fills and reads.  Device memory,
+    which the CPU cannot reach, goes through copies, as in larger calls."""
+    m = binding.Model(model(), "fp32")
+    s, ptr = system(300), binding._ptr
+    call = DeviceCall(host, m, s)
+    host_force = np.zeros((3, s.n))
+    for types, pos, force in ((call.types, ptr(s.pos), ptr(host_force)), (ptr(s.types), call.pos, ptr(host_force)),
+                              (ptr(s.types), ptr(s.pos), call.force)):
+        copied = {p: host.lib.host_copies(p) for p in (call.types, call.pos, call.force)}
+        rc = host.lib.nep_compute(m.h, s.n, types, pos, ptr(s.box), ptr(s.pbc), binding.NEP_HOST, None, None, None, None,
+                                  force, None)
+        binding._check(rc, "nep_compute")
+        for p in copied:
+            assert (host.lib.host_copies(p) > copied[p]) == (p in (types, pos, force))
     host.check()
     m.close()
