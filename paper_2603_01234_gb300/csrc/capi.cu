@@ -239,8 +239,7 @@ struct nep_model {
     int* h_flags = nullptr;        // pinned: maxcnt[2], err
     double* h_totals = nullptr;    // pinned [10 * requests]
     size_t h_totals_cap = 0;
-    double* h_io = nullptr;        // pinned: inputs and outputs of small host calls
-    size_t h_io_cap = 0;           // bytes
+    double* h_io = nullptr;        // pinned, kHostIoBytes: inputs and outputs of small host calls
     unsigned char* h_stage = nullptr;  // pinned staging of the plan tables
     size_t h_stage_cap = 0;
     size_t n_lists = 0;  // particles the lists were sized for
@@ -909,7 +908,7 @@ int copy_totals(nep_model* m, const double* totals, size_t n_req, const TotalsTa
 
 // Particles up to which a host call works on page-locked memory directly.  Measured (water,
 // FP32, whole call): 64 particles 96 us against 127 with copies, 1,000 108 / 136, 4,000
-// 148 / 166; the buffer stays below 0.6 MB.
+// 148 / 166; the buffer takes 0.54 MB.
 constexpr int kDirectMaxN = 4096;
 
 // Whether the CPU may read and write p: device memory among the arrays of a host call takes the
@@ -924,14 +923,14 @@ bool cpu_reaches(const void* p)
     return !p || a.type != cudaMemoryTypeDevice;
 }
 
-int ensure_host_io(nep_model* m, size_t bytes)
+// The buffer has room for the largest such call from the start: growing it would free and
+// allocate page-locked memory (which waits for the device) on calls of rising size, and strand the
+// graphs captured on its address.
+constexpr size_t kHostIoBytes = sizeof(double) * (10 + 16 * (size_t)kDirectMaxN) + sizeof(int) * (size_t)kDirectMaxN;
+
+int ensure_host_io(nep_model* m)
 {
-    if (bytes <= m->h_io_cap) return NEP_OK;
-    if (m->h_io) cudaFreeHost(m->h_io);
-    m->h_io = nullptr;
-    m->h_io_cap = 0;
-    NEP_CUDA(cudaMallocHost((void**)&m->h_io, bytes));
-    m->h_io_cap = bytes;
+    if (!m->h_io) NEP_CUDA(cudaMallocHost((void**)&m->h_io, kHostIoBytes));
     return NEP_OK;
 }
 
@@ -960,8 +959,8 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
         cpu_reaches(virial) && cpu_reaches(site_energy)) {
         // the kernels read the inputs and write the outputs in page-locked memory, each
         // value once: no copies, whose launches would take longer than the transfers
-        const size_t words = 10 + 13 * (size_t)n + 3 * (size_t)n;  // doubles, then n ints
-        NEP_TRY(ensure_host_io(m, sizeof(double) * words + sizeof(int) * (size_t)n));
+        // (totals, 13 n doubles of outputs, 3 n of positions, n ints)
+        NEP_TRY(ensure_host_io(m));
         out = m->h_io;
         double* in = out + 10 + 13 * (size_t)n;
         memcpy(in, pos, sizeof(double) * 3 * (size_t)n);

@@ -245,3 +245,23 @@ def test_small_host_calls_with_device_memory_among_their_arrays(host):
             assert (host.lib.host_copies(p) > copied[p]) == (p in (types, pos, force))
     host.check()
     m.close()
+
+
+def test_small_host_calls_allocate_their_buffer_once(host):
+    """Host calls of rising size keep one page-locked buffer, and a size seen twice before replays
+    its graph after larger ones."""
+    m = binding.Model(model(), "fp32")
+    m.compute(system(4096))
+    before = host.count("malloc_host")
+    for n in (100, 200, 300, 400, 4096):
+        m.compute(system(n))
+    assert host.count("malloc_host") == before
+    m.close()
+    m = binding.Model(model(), "fp32")
+    m.compute(system(100))
+    before = host.count("malloc_host")
+    for n in (200, 300, 400):
+        m.compute(system(n))
+    assert host.count("malloc_host") == before
+    host.check()
+    m.close()
