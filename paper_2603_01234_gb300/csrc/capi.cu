@@ -505,22 +505,27 @@ int ensure_plan_workspace(nep_model* m, const Plan& p)
     return NEP_OK;
 }
 
-// Estimated neighbour counts from the density of the box (first sizing only).
-void initial_capacity(nep_model* m, int n, const double box[3])
+// First estimate of the list capacities: the neighbour counts at the density rho of the box, 30%
+// more and 16.  The box of a configuration with open axes may be far smaller than what its
+// particles would fill, so the estimate has a ceiling; lists that turn out too short grow.  In
+// the FP64 form an angular slot also holds a pair's force (24 bytes): with 512 of them at most the
+// lists and the forces together take no more than two lists of 4,096 and 800 bytes.
+void estimate_capacity(const nep_model* m, double rho, int& radial, int& angular)
 {
-    if (m->mnR > 0 && m->mnA > 0) return;
-    double V = box[0] * box[1] * box[2];
-    double rho = n / V;
     double rR = 0, rA = 0;
     for (double v : m->rcR) rR = std::max(rR, v);
     for (double v : m->rcA) rA = std::max(rA, v);
-    auto est = [&](double rc) {
-        double c = 4.18879 * rc * rc * rc * rho * 1.3 + 16;
-        int k = (int)std::min(c, 4096.0);
-        return (k + 7) & ~7;
+    auto est = [&](double rc, double most) {
+        const double c = 4.18879 * rc * rc * rc * rho * 1.3 + 16;
+        return ((int)std::min(c, most) + 7) & ~7;
     };
-    if (m->mnR <= 0) m->mnR = est(rR);
-    if (m->mnA <= 0) m->mnA = est(rA);
+    if (radial <= 0) radial = est(rR, 4096.0);
+    if (angular <= 0) angular = est(rA, m->precision == NEP_FP64 ? 512.0 : 4096.0);
+}
+
+void initial_capacity(nep_model* m, int n, const double box[3])
+{
+    estimate_capacity(m, n / (box[0] * box[1] * box[2]), m->mnR, m->mnA);
 }
 
 // ---- pipeline stages ----------------------------------------------------------
@@ -2239,15 +2244,7 @@ int nep_request_workspace(nep_model* const* models, int n_models, int model, int
     CellGrid g;
     NEP_TRY(make_grid(models[model], models[model]->rc_max, box, pbc, g));
     int mnR = m->mnR, mnA = m->mnA;
-    if (mnR <= 0 || mnA <= 0) {  // not sized yet: the first-call estimate from the density
-        const double rho = n / (box[0] * box[1] * box[2]);
-        double rR = 0, rA = 0;
-        for (double v : m->rcR) rR = std::max(rR, v);
-        for (double v : m->rcA) rA = std::max(rA, v);
-        auto est = [&](double rc) { return (std::min((int)(4.18879 * rc * rc * rc * rho * 1.3 + 16), 4096) + 7) & ~7; };
-        if (mnR <= 0) mnR = est(rR);
-        if (mnA <= 0) mnA = est(rA);
-    }
+    estimate_capacity(m, n / (box[0] * box[1] * box[2]), mnR, mnA);  // not sized yet: as the first call will
     const size_t rs = m->real_size;
     // cell_of, rec_user, perm_tmp, perm, rec_s, cell_s, cntR, cntA, U, e, force_tmp, partial2
     size_t per_particle = 4 + 4 * rs + 4 + 4 + 4 * rs + 4 + 4 + 4 + rs + rs * Tmax * m->KRP + 24 + 1;

@@ -265,3 +265,26 @@ def test_small_host_calls_allocate_their_buffer_once(host):
     assert host.count("malloc_host") == before
     host.check()
     m.close()
+
+
+def test_fp64_first_sizing_of_a_thin_open_box(host):
+    """The first estimate of the list capacities from the box's density knows nothing of an open
+    axis: a sheet in a flat box is estimated at the ceiling of 4,096.  With the FP64 form's pair
+    forces (24 bytes an angular slot) that is no more memory than two lists of the ceiling and
+    800 bytes a particle, and a configuration that needs more angular slots still gets them."""
+    n = 2000
+    s = system(n, (100.0, 100.0, 0.01))
+    s.pbc[2] = 0
+    m = binding.Model(model(), "fp64")
+    asked = binding.nep_request_workspace([m.h], 0, n, s.box, s.pbc)
+    m.compute(s)
+    radial, angular = binding.nep_get_capacity(m.h)
+    lists = 4 * (radial + angular) + 24 * angular
+    assert radial == 4096 and lists <= 2 * 4 * 4096 + 800
+    others = 600  # records, gradients, totals and staging of a particle: see nep_request_workspace
+    assert binding.nep_workspace_bytes(m.h) <= asked <= n * (lists + others) + 100_000
+    host.set("needA", 1000)
+    m.compute(s)
+    assert binding.nep_get_capacity(m.h)[1] >= 1000
+    host.check()
+    m.close()
