@@ -659,7 +659,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_force_group(EvalArgs<real> a)
         // angular pairs: F_i += f_ij - f_ji, W_i += r_ij (x) f_ji; f_ji is in the slot of j's
         // list that holds i at the opposite cell offset (each code field d + 2 becomes
         // 2 - d).  A pair within rounding of the cutoff may be in one list only; its other
-        // direction is below f_c(r_c - rounding), some 1e-30 of a pair's, and left out.
+        // direction is left out.  The largest term of it is f_c', which falls to zero linearly
+        // at r_c (f_c quadratically): pi^2/2 times the relative distance to r_c, some 1e-15 of a
+        // pair's force, the rounding of the sums that it would enter.
         const int cA = live ? min(a.cntA[i], a.mnA) : 0;
         for (int s = gl; s < cA; s += kG) {
             const uint32_t ea = a.nlA[(size_t)s * n + i];

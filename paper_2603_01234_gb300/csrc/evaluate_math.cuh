@@ -361,11 +361,6 @@ __device__ __forceinline__ void load_grad(const real* p, real* o)
     }
 }
 
-// 1/sqrt(x): the hardware estimate refined by one Newton-Raphson step on
-// f(y) = y^-2 - x, y' = y + y (1 - x y^2) / 2.  The estimate's error has a small
-// consistent sign, which through |u| = |r| / r and the homogeneous harmonics would
-// bias the angular descriptors; after the step the quadratic term is ~1e-14 and
-// what remains is the (unsigned) rounding of y^2.
 // A type pair's n x K coefficient table into registers.  A one-type model's single
 // table starts on a 16-byte boundary and is read with vector loads; several types'
 // tables sit at odd strides (bank spread) and are read as scalars.
@@ -380,6 +375,11 @@ __device__ __forceinline__ void load_coef(const real* c, bool aligned, real (&o)
     }
 }
 
+// 1/sqrt(x): the hardware estimate refined by one Newton-Raphson step on
+// f(y) = y^-2 - x, y' = y + y (1 - x y^2) / 2.  The estimate's error has a small
+// consistent sign, which through r and u = r_ij / r would bias the descriptors of every
+// particle alike; after the step the quadratic term is ~1e-14 and what remains is the
+// (unsigned) rounding of y^2.
 __device__ __forceinline__ float rsqrt_r(float x)
 {
     const float y = rsqrtf(x);

@@ -700,17 +700,6 @@ __device__ __forceinline__ int nbr_images(const CellGrid& g, int cx)
     return hi - lo + 1;
 }
 
-// The distance test: j at the cell offset (dx, dy, dz) from i's cell.  Explicit roundings:
-// every kernel decides alike.
-template <typename real>
-__device__ __forceinline__ real nbr_r2(const PosRec<real>& ri, const PosRec<real>& rj, int dx, int dy, int dz, real lx,
-                                       real ly, real lz)
-{
-    const real x = rj.x - fma(-(real)dx, lx, ri.x), y = rj.y - fma(-(real)dy, ly, ri.y),
-               z = rj.z - fma(-(real)dz, lz, ri.z);
-    return fma(z, z, fma(y, y, x * x));
-}
-
 __device__ __forceinline__ uint32_t nbr_entry(int k, int dx, int dy, int dz)
 {
     return (uint32_t)k | ((uint32_t)((dx + 2) | ((dy + 2) << 3) | ((dz + 2) << 6)) << kJBits);
@@ -800,6 +789,7 @@ __global__ void __launch_bounds__(kBlock) k_neighbors_warp(NeighborArgs<real> a)
                 for (int p = p0; p < p1; ++p) {
                     const PosRec<real> ri = recs[warp][p];
                     const int i = first + p;
+                    // the distance test of k_neighbors, with its roundings: both decide alike
                     const real x = rj.x - fma(-ox, lx, ri.x), y = rj.y - fma(-oy, ly, ri.y), z = rj.z - fma(-oz, lz, ri.z);
                     const real r2 = fma(z, z, fma(y, y, x * x));
                     real cR = cR1, cA = cA1;
