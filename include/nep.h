@@ -355,7 +355,10 @@ int nep_compute_static(nep_model* m, int n, const int32_t* types, const double* 
                        double* site_energy, double* force, double* virial);
 
 /*
- * Autotuner.  The FP32 descriptor kernel is compiled in variants that keep 2 or 3
+ * Autotuner.  Larger FP32 evaluations (from some 10,000 to 25,000 particles on, depending on
+ * the model) run one thread per particle; the smaller ones and FP64 run kernels that have no
+ * variants, and for them nep_autotune returns the variants in use and nep_set_tuning
+ * has no effect until a larger evaluation.  The descriptor kernel is compiled in variants that keep 2 or 3
  * thread blocks resident per SM, and the radial-force kernel in variants that keep
  * 3, 4 or 5 resident (a register budget per thread) and walk the neighbour list in
  * groups of 4 or 8 entries (the next group's entries load while the current group

@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "dispatch.h"
 #include "nep.h"
 #include "nep_common.cuh"
 
@@ -159,9 +160,10 @@ struct Plan {
     std::vector<unsigned char> models;  // ModelDesc<real> entries, raw bytes
     int n = 0, ncell = 0, n_models = 0;
     int n_cap = 0, items_cap = 0, ncell_cap = 0, req_cap = 0;
-    int Tmax = 1;
+    int Tmax = 1, Hmax = 1;
     double *energy = nullptr, *virial_total = nullptr;  // where the kernels write the caller's totals (or null)
     size_t smem_desc = 0, smem_force = 0, smem_nbr = 0;
+    NeighborLoad nbr;
     std::vector<unsigned char> key;     // identity of the uploaded tables
     Buf dev;                            // [counts | reqs | items | models] on the device
     size_t off_reqs = 0, off_items = 0, off_models = 0;
@@ -335,16 +337,19 @@ void set_models(Plan& p, nep_model* const* models, int n_models)
 {
     p.n_models = n_models;
     p.models.resize(sizeof(ModelDesc<real>) * n_models);
-    p.Tmax = 1;
+    p.Tmax = p.Hmax = 1;
     p.smem_desc = p.smem_force = p.smem_nbr = 0;
     for (int k = 0; k < n_models; ++k) {
         ModelDesc<real> d = model_desc<real>(models[k]);
         memcpy(p.models.data() + k * sizeof d, &d, sizeof d);
         p.Tmax = std::max(p.Tmax, models[k]->T);
+        p.Hmax = std::max(p.Hmax, models[k]->H);
         p.smem_desc = std::max(p.smem_desc, models[k]->smem_desc);
         p.smem_force = std::max(p.smem_force, models[k]->smem_force);
         p.smem_nbr = std::max(p.smem_nbr, neighbor_smem<real>(models[k]->T));
     }
+    p.nbr = NeighborLoad();
+    for (const ReqInfo& r : p.reqs) p.nbr.add(r.g, r.n, models[r.model]->T);
 }
 
 constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -575,7 +580,13 @@ int run_kick_drift_cells(nep_model* m, const Plan& p, const int* types_d, const 
 
 int plan_form(const nep_model* m, const Plan& p)
 {
-    return neighbor_form(p.items_cap, p.n, p.ncell, m->precision == NEP_FP64);
+    return neighbor_form(p.nbr, m->precision == NEP_FP64);
+}
+
+bool plan_by_groups(const nep_model* m, const Plan& p, bool virial)
+{
+    return evaluate_by_groups({p.n_cap, p.items_cap, p.Tmax, p.Hmax, m->mnR, m->mnA, p.smem_desc, virial},
+                              m->precision == NEP_FP64);
 }
 
 template <typename real>
@@ -660,8 +671,9 @@ int run_evaluate(nep_model* m, const Plan& p, double* force, double* virial, dou
         a.kick_half_dt = kick->half_dt;
         for (int t = 0; t < kMdMaxTypes; ++t) a.kick_im.v[t] = t < m->T ? kick->inv_m_acc[t] : 0.0;
     }
-    cudaError_t e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, p.items_cap, p.smem_desc,
-                                          p.smem_force, m->cur, mid, m->mb_desc, m->mb_force, m->ch_force);
+    cudaError_t e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, p.items_cap,
+                                          plan_by_groups(m, p, virial != nullptr), p.smem_desc, p.smem_force, m->cur,
+                                          mid, m->mb_desc, m->mb_force, m->ch_force);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("evaluate: ") + cudaGetErrorString(e));
     return NEP_OK;
 }
@@ -754,7 +766,7 @@ std::vector<unsigned char> eval_graph_key(const nep_model* m, const Plan& p, con
     };
     const int ints[] = {p.n_cap, p.items_cap, p.ncell_cap, p.Tmax, m->mnR, m->mnA, m->mb_desc, m->mb_force, m->ch_force,
                         m->eval_per_bead ? 1 : 0, m->precision, m->MBT, (int)sizeof(real),
-                        plan_form(m, p)};
+                        plan_form(m, p), plan_by_groups(m, p, m->eval_per_bead) ? 1 : 0};
     put(ints, sizeof ints);
     const size_t sm[] = {p.smem_desc, p.smem_force, p.smem_nbr, p.off_reqs, p.off_items, p.off_models};
     put(sm, sizeof sm);
@@ -1055,7 +1067,7 @@ struct TuneEvents {
 template <typename real>
 int autotune_plan(nep_model* m, const Plan& p, double* force_d)
 {
-    if (evaluate_by_groups(p.items_cap, m->precision == NEP_FP64)) return NEP_OK;  // no variants
+    if (plan_by_groups(m, p, false)) return NEP_OK;  // no variants
     TuneEvents ev;
     for (cudaEvent_t& x : ev.e) NEP_CUDA(cudaEventCreate(&x));
     cudaEvent_t e0 = ev.e[0], em = ev.e[1], e1 = ev.e[2];
@@ -2480,7 +2492,9 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     na.maxcnt = flags;
     na.accF = sizeof(real) == 4 ? acc_force(base + L.acc) : nullptr;
     na.accW = sizeof(real) == 4 && virial ? acc_virial(base + L.acc, n) : nullptr;
-    e = launch_neighbors<real>(na, n_items, neighbor_form(n_items, n, g.ncell, sizeof(real) == 8), neighbor_smem<real>(m->T), m->cur);
+    NeighborLoad load;
+    load.add(g, n, m->T);
+    e = launch_neighbors<real>(na, n_items, neighbor_form(load, sizeof(real) == 8), neighbor_smem<real>(m->T), m->cur);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("neighbours: ") + cudaGetErrorString(e));
     EvalArgs<real> a;
     a.n = n;
@@ -2514,8 +2528,10 @@ int compute_static_impl(nep_model* m, int n, const int32_t* types, const double*
     a.icounter = counters + 4;
     a.err = flags + 2;
     a.totals = totals;
-    e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, n_items, m->smem_desc, m->smem_force, m->cur, nullptr,
-                              m->mb_desc, m->mb_force, m->ch_force);
+    const bool groups = evaluate_by_groups({n, n_items, m->T, m->H, a.mnR, a.mnA, m->smem_desc, virial != nullptr},
+                                           sizeof(real) == 8);
+    e = launch_evaluate<real>(m->nR, m->nA, m->KR, m->KA, a, n_items, groups, m->smem_desc, m->smem_force, m->cur,
+                              nullptr, m->mb_desc, m->mb_force, m->ch_force);
     if (e != cudaSuccess) return fail(NEP_ERR_CUDA, std::string("evaluate: ") + cudaGetErrorString(e));
     NEP_TRY(copy_totals(m, totals, 1, to_energy, to_virial));
     // the handle's pinned status buffer (allocated by nep_create) receives the words

@@ -637,24 +637,12 @@ static cudaError_t launch_force_radial(const EvalArgs<float>& a, int nb, size_t 
     return launch_k(k_force_radial<float, NR, KR, 3, 4>, nb, kBlock, smem, st, a);
 }
 
-// FP32 batches up to this many work items run the group kernels (evaluate_group.cu).  Theirs
-// is the shorter latency, the thread-per-particle kernels' the fewer instructions: on
-// water the group kernels' two launches take 37 us at 4 items (82 us here), 50 at 24 (104)
-// and then 0.53 us an item, and the ones here about 110 us until the chip is full at 456
-// items.  FP64 always runs the group kernels: bound by the FP64 pipe, they evaluate each
-// ordered angular pair once and do not spill (100,000-bead water 5.01 ms; one thread per
-// particle and both directions of each pair took 7.00 ms).
-constexpr int kGroupMaxItems = 200;
-
-bool evaluate_by_groups(int items_cap, bool fp64) { return fp64 || items_cap <= kGroupMaxItems; }
-
 template <typename real>
-cudaError_t launch_evaluate(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap, size_t smem_desc,
-                            size_t smem_force, cudaStream_t st, cudaEvent_t mid, int mb_desc, int mb_force,
-                            int ch_force)
+cudaError_t launch_evaluate(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap, bool by_groups,
+                            size_t smem_desc, size_t smem_force, cudaStream_t st, cudaEvent_t mid, int mb_desc,
+                            int mb_force, int ch_force)
 {
-    if (evaluate_by_groups(items_cap, sizeof(real) == 8))
-        return launch_evaluate_group<real>(nR, nA, KR, KA, a, items_cap, st, mid);
+    if (by_groups) return launch_evaluate_group<real>(nR, nA, KR, KA, a, items_cap, st, mid);
     if constexpr (sizeof(real) == 4) {
         if (!a.accF || !a.wsum) return cudaErrorInvalidValue;  // the FP32 form scatters into a.accF
         const int nb = items_cap;
@@ -675,7 +663,7 @@ cudaError_t launch_evaluate(int nR, int nA, int KR, int KA, const EvalArgs<real>
 #define NEP_INSTANTIATE(real)                                                                             \
     template bool evaluate_shape_supported<real>(int, int, int, int);                                     \
     template cudaError_t evaluate_set_smem<real>(int, int, int, int, size_t, size_t);                     \
-    template cudaError_t launch_evaluate<real>(int, int, int, int, const EvalArgs<real>&, int, size_t, size_t, \
+    template cudaError_t launch_evaluate<real>(int, int, int, int, const EvalArgs<real>&, int, bool, size_t, size_t, \
                                                cudaStream_t, cudaEvent_t, int, int, int);
 NEP_INSTANTIATE(float)
 NEP_INSTANTIATE(double)

@@ -821,18 +821,6 @@ __global__ void __launch_bounds__(kBlock) k_neighbors_warp(NeighborArgs<real> a)
     }
 }
 
-// Which kernel.  Measured (FP32; one warp per particle / per eight particles / one thread per
-// particle): water at 4 items 14 / 30 / 48 us, at 24 items 19 / 39 / 67, at 782 items
-// 254 / 130 / 103; a 60,000-particle nanowire (469 items, a dense core) 122 / 69 / 104; a
-// 50,000-particle monolayer (392 items, 1.2 particles to a cell, so that nothing is
-// shared between a warp's particles) 73 / 36 / 25.  FP64 tests every pair in FP64 in the warp
-// kernels and screens in FP32 in the other (782 items: 1217 / 1034 / 223 us).
-int neighbor_form(int items_cap, int n, int ncell, bool fp64)
-{
-    if (items_cap <= 90) return 1;
-    return !fp64 && items_cap <= 512 && n >= 2 * ncell ? 8 : 0;
-}
-
 // FP64 form: the FP32 copies of the sorted records that screen the distance tests
 // of k_neighbors (one conversion per particle instead of per candidate)
 __global__ void __launch_bounds__(kBlock) k_round_records(const PlanCounts* __restrict__ pc,

@@ -310,23 +310,17 @@ cudaError_t launch_kick_drift_bin(const PlanCounts* counts, int items_cap, const
                                   double* vel, const double* force, int* cell_of, PosRec<real>* rec_user,
                                   int* cell_count, int* err, cudaStream_t st);
 
-// The neighbour kernel of a batch of n particles in ncell cells: the particles that a warp
-// takes (1 or 8), or 0 for one thread per particle.
-int neighbor_form(int items_cap, int n, int ncell, bool fp64);
-
+// form: the particles that a warp takes (1 or 8), or 0 for one thread per particle (dispatch.h).
 template <typename real>
 cudaError_t launch_neighbors(const NeighborArgs<real>& a, int items_cap, int form, size_t smem, cudaStream_t st);
 
-// Shape-dispatched evaluation; returns cudaErrorInvalidValue for an uncompiled shape.
-// mb_desc / mb_force / ch_force: the variants of the thread-per-particle kernels
-// (resident blocks per SM, walk chunk), which evaluate_by_groups says are not used.
+// Shape-dispatched evaluation by the group kernels or one thread per particle (FP32 only);
+// returns cudaErrorInvalidValue for an uncompiled shape.  mb_desc / mb_force / ch_force:
+// the variants of the thread-per-particle kernels (resident blocks per SM, walk chunk).
 template <typename real>
-cudaError_t launch_evaluate(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap, size_t smem_desc,
-                            size_t smem_force, cudaStream_t st, cudaEvent_t mid = nullptr, int mb_desc = 3,
-                            int mb_force = 3, int ch_force = 4);
-
-// Whether a batch of items_cap work items runs the group kernels (which have no variants).
-bool evaluate_by_groups(int items_cap, bool fp64);
+cudaError_t launch_evaluate(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap, bool by_groups,
+                            size_t smem_desc, size_t smem_force, cudaStream_t st, cudaEvent_t mid = nullptr,
+                            int mb_desc = 3, int mb_force = 3, int ch_force = 4);
 
 template <typename real>
 cudaError_t launch_evaluate_group(int nR, int nA, int KR, int KA, const EvalArgs<real>& a, int items_cap,

@@ -160,9 +160,6 @@ cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.
 
 namespace nep {
 
-int neighbor_form(int, int, int, bool) { return 1; }
-bool evaluate_by_groups(int, bool) { return true; }
-
 template <typename real>
 cudaError_t launch_cell_build(const PlanCounts* pc, int n_cap, int, int ncell_cap, bool zero_counts, bool, const WorkItem*,
                               const ReqInfo*, const ModelDesc<real>*, const double* pos, const int* types, int* cell_of,
@@ -213,7 +210,7 @@ cudaError_t launch_neighbors(const NeighborArgs<real>& a, int, int, size_t, cuda
 }
 
 template <typename real>
-cudaError_t launch_evaluate(int, int, int, int, const EvalArgs<real>& a, int items_cap, size_t, size_t,
+cudaError_t launch_evaluate(int, int, int, int, const EvalArgs<real>& a, int items_cap, bool, size_t, size_t,
                             cudaStream_t st, cudaEvent_t, int, int, int)
 {
     ++counters["evaluate"];
@@ -259,7 +256,7 @@ cudaError_t launch_cg_map(int, int, const int*, const int*, const double*, const
                                                      double, double*, double*, const double*, int*, PosRec<real>*, int*,  \
                                                      int*, cudaStream_t);                                                 \
     template cudaError_t launch_neighbors<real>(const NeighborArgs<real>&, int, int, size_t, cudaStream_t);               \
-    template cudaError_t launch_evaluate<real>(int, int, int, int, const EvalArgs<real>&, int, size_t, size_t,            \
+    template cudaError_t launch_evaluate<real>(int, int, int, int, const EvalArgs<real>&, int, bool, size_t, size_t,      \
                                                cudaStream_t, cudaEvent_t, int, int, int);                                 \
     template bool evaluate_shape_supported<real>(int, int, int, int);                                                     \
     template cudaError_t evaluate_set_smem<real>(int, int, int, int, size_t, size_t);
@@ -276,6 +273,23 @@ void host_set(const char* what, long value)
     else if (w == "fail_host_in") fail_host_in = value;
     else if (w == "needR") needR = (int)value;
     else if (w == "needA") needA = (int)value;
+}
+// the rules of dispatch.h: the neighbour kernel of count boxes of n particles, and whether a batch
+// runs the group kernels
+int host_neighbor_form(int boxes, const int* n, const int* types, const double* box, const int* pbc, const double* rc,
+                       int fp64)
+{
+    NeighborLoad w;
+    for (int r = 0; r < boxes; ++r) {
+        CellGrid g;
+        if (make_grid(nullptr, rc[r], box + 3 * r, pbc + 3 * r, g) != NEP_OK) return -1;
+        w.add(g, n[r], types[r]);
+    }
+    return neighbor_form(w, fp64 != 0);
+}
+int host_by_groups(int n, int items, int types, int hidden, int mnR, int mnA, int table_bytes, int virial, int fp64)
+{
+    return evaluate_by_groups({n, items, types, hidden, mnR, mnA, (size_t)table_bytes, virial != 0}, fp64 != 0);
 }
 // memory of the stand-in device (kind 2), of another device that kernels do not reach (3), or
 // page-locked memory (1)

@@ -8,7 +8,7 @@ from paper_2603_01234_gb300 import binding, inputs
 from tests.gpu_common import monolayer_model, small_systems, water_model
 
 pytestmark = pytest.mark.gpu
-ITEMS = 600  # work items beyond the group kernels' (at most 200) and the warp kernels' (at most 512)
+PARTICLES = 70_000  # beyond every rule's line for the group and the warp kernels (dispatch.h)
 
 
 @pytest.mark.parametrize("name", ["water", "monolayer"])
@@ -44,7 +44,7 @@ def test_small_systems_in_a_large_batch(nep_lib, case):
     name, model, system = case
     h = binding.Model(model, "fp32")
     alone = h.compute(system)
-    copies = ITEMS // -(-system.n // 128) + 1
+    copies = PARTICLES // system.n + 1
     req_n, req_box, req_pbc, types, pos = binding.pack_requests([system] * copies)
     n = int(req_n.sum())
     e, wt, U, F, W = np.zeros(copies), np.zeros((copies, 9)), np.zeros(n), np.zeros(3 * n), np.zeros(9 * n)

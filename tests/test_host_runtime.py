@@ -288,3 +288,52 @@ def test_fp64_first_sizing_of_a_thin_open_box(host):
     assert binding.nep_get_capacity(m.h)[1] >= 1000
     host.check()
     m.close()
+
+
+def neighbor_form(host, boxes, fp64=False):
+    """boxes: (particles, box, pbc, types, r_c) of each request."""
+    arr = lambda k, t: np.ascontiguousarray([b[k] for b in boxes], t)  # noqa: E731
+    n, box, pbc, types, rc = arr(0, np.int32), arr(1, np.float64), arr(2, np.int32), arr(3, np.int32), arr(4, np.float64)
+    p = binding._ptr
+    return host.lib.host_neighbor_form(len(boxes), p(n), p(types), p(box), p(pbc), p(rc), int(fp64))
+
+
+def water(n, types=1):
+    return n, [(n / 0.0334) ** (1 / 3)] * 3, [1, 1, 1], types, 8.0
+
+
+def monolayer(n):
+    s = inputs.monolayer(max(2, round((n / 4) ** 0.5)), max(2, round(n / 4 / max(2, round((n / 4) ** 0.5)))))
+    return s.n, s.box, s.pbc, 4, 15.0
+
+
+def test_neighbour_kernel_of_a_batch(host):
+    """The kernel that measured fastest (or within a few percent of it) at sizes where the choice
+    costs most."""
+    for n, want in ((2_000, 1), (9_000, 1), (30_000, 8), (50_000, 0), (60_000, 0), (100_000, 0)):
+        assert neighbor_form(host, [water(n)]) == want, n
+    for n, want in ((9_000, 1), (30_000, 8), (58_000, 8), (77_000, 0)):
+        assert neighbor_form(host, [water(n, types=2)]) == want, n
+    assert neighbor_form(host, [monolayer(50_000)]) == 0 and neighbor_form(host, [monolayer(4_000)]) == 1
+    wire = inputs.nanowire(60_001, n_cells_x=196)
+    assert neighbor_form(host, [(wire.n, wire.box, wire.pbc, 3, 7.0)]) == 8
+    # batches: what counts is the densest request's tests against everyone's
+    assert neighbor_form(host, [water(100)] * 250) == 0 and neighbor_form(host, [water(100)] * 60) == 1
+    rng = np.random.default_rng(7)
+    sizes = np.exp(rng.uniform(np.log(64), np.log(1000), 100)).astype(int)
+    assert neighbor_form(host, [water(n) if k % 2 else monolayer(n) for k, n in enumerate(sizes)]) == 1
+    assert neighbor_form(host, [water(11_000)], fp64=True) == 1 and neighbor_form(host, [water(12_000)], fp64=True) == 0
+
+
+@pytest.mark.parametrize("n,items,types,hidden,mnR,mnA,table_kb,virial,want", [
+    (9_000, 71, 1, 30, 112, 40, 6, 1, 1), (16_000, 125, 1, 30, 136, 48, 6, 0, 0), (60_000, 469, 1, 30, 136, 48, 6, 1, 0),
+    (16_000, 125, 4, 50, 24, 24, 43, 0, 0), (25_600, 200, 4, 50, 24, 24, 43, 1, 0),  # monolayer
+    (25_600, 400, 4, 50, 24, 24, 43, 1, 0), (12_288, 96, 4, 50, 24, 24, 43, 1, 1),
+    (25_600, 200, 3, 40, 128, 64, 26, 0, 1), (60_001, 469, 3, 40, 128, 64, 26, 1, 0),  # nanowire
+    (20_000, 157, 1, 30, 328, 112, 6, 1, 1),  # many pairs
+    (12_000, 94, 1, 700, 112, 40, 134, 1, 0), (9_500, 75, 1, 700, 112, 40, 134, 1, 1),  # a wide layer
+    (25_600, 200, 1, 700, 112, 40, 134, 0, 1), (12_000, 94, 2, 300, 112, 40, 104, 0, 0)])
+def test_evaluation_kernels_of_a_batch(host, n, items, types, hidden, mnR, mnA, table_kb, virial, want):
+    args = (n, items, types, hidden, mnR, mnA, table_kb * 1024, virial)
+    assert host.lib.host_by_groups(*args, 0) == want
+    assert host.lib.host_by_groups(*args, 1) == 1  # FP64
