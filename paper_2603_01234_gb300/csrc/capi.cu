@@ -972,8 +972,7 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
     double *force_d = force, *virial_d = virial, *site_d = site_energy;
     double* totals = m->totals.as<double>();
     double* out = nullptr;  // a small host call's outputs in pinned memory: totals, force, virial, site energies
-    if (mem == NEP_HOST && n <= kDirectMaxN && cpu_reaches(types) && cpu_reaches(pos) && cpu_reaches(force) &&
-        cpu_reaches(virial) && cpu_reaches(site_energy)) {
+    if (mem == NEP_HOST && n <= kDirectMaxN && cpu_reaches(types) && cpu_reaches(pos)) {
         // the kernels read the inputs and write the outputs in page-locked memory, each
         // value once: no copies, whose launches would take longer than the transfers
         // (totals, 13 n doubles of outputs, 3 n of positions, n ints)
@@ -1011,6 +1010,7 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
     } else if (!force_d) {
         force_d = m->force_tmp.as<double>();
     }
+    bool cpu_force = true, cpu_virial = true, cpu_site = true;  // which outputs of a direct host call the CPU fills
     // one synchronisation per call: the evaluation, its outputs and its status words
     // are enqueued together; lists that overflowed are grown and the call runs again
     for (int attempt = 0;; ++attempt) {
@@ -1024,6 +1024,11 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
             NEP_CUDA(cudaMemcpyAsync(m->h_totals, totals, sizeof(double) * 10, cudaMemcpyDeviceToHost, m->cur));
         }
         NEP_TRY(copy_totals(m, totals, 1, to_energy, to_virial));
+        if (out) {  // while the GPU works
+            cpu_force = cpu_reaches(force);
+            cpu_virial = cpu_reaches(virial);
+            cpu_site = cpu_reaches(site_energy);
+        }
         NEP_TRY(leave(m, stream));
         bool retry = false;
         NEP_TRY(eval_status(m, retry));
@@ -1037,9 +1042,14 @@ int compute_impl(nep_model* m, int n, const int32_t* types, const double* pos, c
         if (virial_total)
             for (int k = 0; k < 9; ++k) virial_total[k] = t[1 + k];
         if (out) {
-            if (force) memcpy(force, force_d, sizeof(double) * 3 * (size_t)n);
-            if (virial) memcpy(virial, virial_d, sizeof(double) * 9 * (size_t)n);
-            if (site_energy) memcpy(site_energy, site_d, sizeof(double) * (size_t)n);
+            auto give = [&](double* to, const double* from, size_t per, bool cpu) -> int {
+                if (to && cpu) memcpy(to, from, sizeof(double) * per * (size_t)n);
+                else if (to) NEP_CUDA(cudaMemcpy(to, from, sizeof(double) * per * (size_t)n, cudaMemcpyDefault));
+                return NEP_OK;
+            };
+            NEP_TRY(give(force, force_d, 3, cpu_force));
+            NEP_TRY(give(virial, virial_d, 9, cpu_virial));
+            NEP_TRY(give(site_energy, site_d, 1, cpu_site));
         }
     }
     return NEP_OK;

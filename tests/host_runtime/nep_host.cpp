@@ -119,7 +119,13 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p)
 }
 cudaError_t cudaMemset(void* p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t st) { return enqueue(st, [=] { memset(p, v, n); }); }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind)
+{
+    ++copies[d];
+    ++copies[s];
+    memcpy(d, s, n);
+    return cudaSuccess;
+}
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st)
 {
     ++copies[d];
