@@ -629,6 +629,8 @@ __device__ __forceinline__ void reduce_totals(double (&v)[10], int item, const W
     __shared__ double part[10][12];
     __shared__ bool last;
     const int t = threadIdx.x;
+    // the caller's addresses, loaded here so that the last block does not wait for them
+    double *const energy = counts->energy, *const virial = counts->virial;
 #pragma unroll
     for (int k = 0; k < 10; ++k) red[k][t] = v[k];
     __syncthreads();
@@ -659,7 +661,7 @@ __device__ __forceinline__ void reduce_totals(double (&v)[10], int item, const W
     const double gs = sum_partials(partial + (size_t)g0 * 10, gn, 1, part);
     const int ng = (n_items + kGroup - 1) / kGroup;
     if (ng == 1) {  // one group: its sum is the total
-        if (t < 10) write_total(*counts, totals, it.req, t, gs);
+        if (t < 10) write_total(energy, virial, totals, it.req, t, gs);
         if (t == 0) gcounter[g0] = 0u;
         return;
     }
@@ -674,7 +676,7 @@ __device__ __forceinline__ void reduce_totals(double (&v)[10], int item, const W
     if (!last) return;
     __threadfence();
     const double ts = sum_partials(partial + (size_t)rq.item_begin * 10, ng, kGroup, part);
-    if (t < 10) write_total(*counts, totals, it.req, t, ts);
+    if (t < 10) write_total(energy, virial, totals, it.req, t, ts);
     if (t == 0) counter[it.req] = 0u;
 }
 

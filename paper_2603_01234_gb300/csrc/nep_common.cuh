@@ -231,12 +231,13 @@ constexpr int kGroup = 32;
 // touching memory out of bounds.
 constexpr int kErrCellList = 4;
 
-// Total t (E, then W[9]) of request r: into all [requests][10] and the caller's own arrays.
-__device__ __forceinline__ void write_total(const PlanCounts& pc, double* all, int r, int t, double v)
+// Total t (E, then W[9]) of request r: into all [requests][10] and the caller's own arrays (either
+// may be null).
+__device__ __forceinline__ void write_total(double* energy, double* virial, double* all, int r, int t, double v)
 {
     all[(size_t)r * 10 + t] = v;
-    if (pc.energy && t == 0) pc.energy[r] = v;
-    if (pc.virial && t > 0) pc.virial[(size_t)r * 9 + t - 1] = v;
+    if (energy && t == 0) energy[r] = v;
+    if (virial && t > 0) virial[(size_t)r * 9 + t - 1] = v;
 }
 
 template <typename real>

@@ -235,7 +235,7 @@ cudaError_t launch_evaluate(int, int, int, int, const EvalArgs<real>& a, int ite
         if ((uintptr_t)a.counts->energy % 8 || (uintptr_t)a.counts->virial % 8) ++counters["bad"];
         if (counters["bad"]) return;
         for (size_t r = 0; r < nq; ++r)  // energy r + 0.5, virial component k r + k
-            for (int t = 0; t < 10; ++t) write_total(*a.counts, a.totals, (int)r, t, (double)r + (t ? t - 1 : 0.5));
+            for (int t = 0; t < 10; ++t) write_total(a.counts->energy, a.counts->virial, a.totals, (int)r, t, (double)r + (t ? t - 1 : 0.5));
     });
 }
 
