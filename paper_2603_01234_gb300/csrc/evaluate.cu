@@ -119,14 +119,11 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
             real g = real(0);
 #pragma unroll
             for (int k = 0; k < KR; ++k) g += c[nn * KR + k] * fs[k];
-            if constexpr (sizeof(real) == 4) {  // plus the coefficients' FP32 rounding residuals
-                const real* cl = P + off.cRl;
-                real gl = real(0);
+            const real* cl = P + off.cRl;  // plus the coefficients' FP32 rounding residuals
+            real gl = real(0);
 #pragma unroll
-                for (int k = 0; k < KR; ++k) gl += cl[nn * KR + k] * fs[k];
-                g += gl;
-            }
-            q[nn] = g;
+            for (int k = 0; k < KR; ++k) gl += cl[nn * KR + k] * fs[k];
+            q[nn] = g + gl;
         }
     } else {
 #pragma unroll 1
@@ -217,14 +214,13 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
         // separate accumulators, so the energy is that of the caller's FP64 weights;
         // the gradient (forces, whose tolerance is far looser) uses the FP32 weights.
         // BF16 weights W0 are FP32 numbers already and have no residual table.
-        constexpr bool kRes = sizeof(real) == 4;
         constexpr bool res0 = RES == 1;
         const real* b0 = P + off.b0 + ti * H;
         const real* w1 = P + off.w1 + ti * H;
-        const real* b0l = P + (kRes ? off.b0l : off.b0) + ti * H;
-        const real* w1l = P + (kRes ? off.w1l : off.w1) + ti * H;
+        const real* b0l = P + off.b0l + ti * H;
+        const real* w1l = P + off.w1l + ti * H;
         U = -P[off.b1 + ti];
-        real Ul = kRes ? -P[off.b1l + ti] : real(0);
+        real Ul = -P[off.b1l + ti];
 #pragma unroll
         for (int v = 0; v < ND; ++v) dq[v] = real(0);
         if (T == 1) {
@@ -240,22 +236,20 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
                 real x = -b0[mu];
 #pragma unroll
                 for (int v = 0; v < ND; ++v) x += w[v] * q[v];
-                if constexpr (kRes) {  // residual row four entries at a time (vector loads)
-                    real xl = -b0l[mu];
-                    if constexpr (res0)
+                real xl = -b0l[mu];  // the residual row four entries at a time (vector loads)
+                if constexpr (res0)
 #pragma unroll
-                        for (int v4 = 0; v4 < NDV; v4 += 4) {
-                            real wl[4];
-                            load4(w0l + mu * NDV + v4, wl);
+                    for (int v4 = 0; v4 < NDV; v4 += 4) {
+                        real wl[4];
+                        load4(w0l + mu * NDV + v4, wl);
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (v4 + u < ND) xl += wl[u] * q[v4 + u];
-                        }
-                    x += xl;
-                }
+                        for (int u = 0; u < 4; ++u)
+                            if (v4 + u < ND) xl += wl[u] * q[v4 + u];
+                    }
+                x += xl;
                 const real h = tanh_r(x);
                 U += w1[mu] * h;
-                if constexpr (kRes) Ul += w1l[mu] * h;
+                Ul += w1l[mu] * h;
                 const real coef = w1[mu] * fma(-h, h, real(1));
 #pragma unroll
                 for (int v = 0; v < ND; ++v) dq[v] += coef * w[v];
@@ -269,22 +263,20 @@ __device__ __forceinline__ void descriptor_item(const EvalArgs<real>& a, const W
                 real x = -b0[mu];
 #pragma unroll
                 for (int v = 0; v < ND; ++v) x += w0[mu * ND + v] * q[v];
-                if constexpr (kRes) {
-                    real xl = -b0l[mu];
-                    if constexpr (res0)
+                real xl = -b0l[mu];
+                if constexpr (res0)
 #pragma unroll
-                        for (int v = 0; v < ND; ++v) xl += w0l[mu * ND + v] * q[v];
-                    x += xl;
-                }
+                    for (int v = 0; v < ND; ++v) xl += w0l[mu * ND + v] * q[v];
+                x += xl;
                 const real h = tanh_r(x);
                 U += w1[mu] * h;
-                if constexpr (kRes) Ul += w1l[mu] * h;
+                Ul += w1l[mu] * h;
                 const real coef = w1[mu] * fma(-h, h, real(1));
 #pragma unroll
                 for (int v = 0; v < ND; ++v) dq[v] += coef * w0[mu * ND + v];
             }
         }
-        if constexpr (kRes) U += Ul;
+        U += Ul;
     }
     a.U[i] = U;
     // e_i^t[k] = sum_n dU/dq_n c^{t_i t}_{nk}
