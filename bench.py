@@ -44,10 +44,10 @@ FLOPS_PEAK_NOTE = "FP32 ALU peak = SMs (device-reported) x 128 FP32 lanes x 2 fl
 # DRAM bytes per particle of one launch of the dominant kernel, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum); valid only for the evaluate.cu
 # source it was taken on, otherwise the bench reports traffic as null.
-KERNEL_TRAFFIC = {"evaluate_cu_sha1": "d2c4d44fa96296386a005caeb16897c4dc11cf15", "bytes_per_particle": 454.2,
+KERNEL_TRAFFIC = {"evaluate_cu_sha1": "3011cca39ae776772cc5607dde11d7e66be00c12", "bytes_per_particle": 453.3,
                   "kernel": "descriptor_network",
-                  "capture": "ncu --set full, k_descriptor (descriptor + network + angular forces), 100,000-bead water, "
-                             "variants 3,3,4, cold caches: 45.31 MB read + 0.11 MB written per launch"}
+                  "capture": "ncu, k_descriptor (descriptor + network + angular forces), 100,000-bead water, "
+                             "variants 3,3,4, cold caches: 45.31 MB read + 0.01 MB written per launch"}
 
 
 N_BEADS = 100_000

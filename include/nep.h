@@ -355,18 +355,19 @@ int nep_compute_static(nep_model* m, int n, const int32_t* types, const double* 
                        double* site_energy, double* force, double* virial);
 
 /*
- * Autotuner.  Larger FP32 evaluations (from some 10,000 to 25,000 particles on, depending on
- * the model) run one thread per particle; the smaller ones and FP64 run kernels that have no
- * variants, and for them nep_autotune returns the variants in use and nep_set_tuning
- * has no effect until a larger evaluation.  The descriptor kernel is compiled in variants that keep 2 or 3
- * thread blocks resident per SM, and the radial-force kernel in variants that keep
- * 3, 4 or 5 resident (a register budget per thread) and walk the neighbour list in
- * groups of 4 or 8 entries (the next group's entries load while the current group
- * is evaluated).  nep_autotune evaluates the configuration several times with each
- * variant, times the two kernels separately with CUDA events, and keeps for each
- * kernel its default (3 blocks; groups of 4) unless another variant is at least 5%
- * faster; the first nep_md_step of a new configuration shape (n and cell grid) does
- * the same unless disabled.  All variants give identical results.  Inputs as in
+ * Autotuner.  Larger FP32 evaluations (from some 10,000 to 25,000 particles on,
+ * depending on the model) run one thread per particle.  The smaller ones and FP64 run
+ * kernels that have no variants: for them nep_autotune returns the variants in use,
+ * and nep_set_tuning has no effect until a larger evaluation.  The descriptor kernel
+ * is compiled in variants that keep 2 or 3 thread blocks resident per SM, and the
+ * radial-force kernel in variants that keep 3, 4 or 5 resident (a register budget
+ * per thread) and walk the neighbour list in groups of 4 or 8 entries (the next
+ * group's entries load while the current group is evaluated).  nep_autotune
+ * evaluates the configuration several times with each variant, times the two kernels
+ * separately with CUDA events, and keeps for each kernel its default (3 blocks;
+ * groups of 4) unless another variant is at least 5% faster; the first nep_md_step
+ * of a new configuration shape (n and cell grid) does the same unless disabled.  All
+ * variants give identical results.  Inputs as in
  * nep_compute; the chosen variants are returned (any output may be NULL).
  */
 int nep_autotune(nep_model* m, int n, const int32_t* types, const double* pos, const double box[3],
